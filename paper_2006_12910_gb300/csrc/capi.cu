@@ -212,7 +212,7 @@ void fill_dom(DomDev& D, const lbm_params& p, int kind) {
               (p.inlet_outlet ? FLAG_IO : 0);
     D.V = store_vector_width(kind);
     D.pitch = (int32_t)round_up(p.nx, std::max<int64_t>(D.V, 128 / (int64_t)elem_bytes(kind)));
-    // y walls: one ghost row on each side of every plane (bounce-back mailboxes)
+    // y walls: one ghost row on each side of every plane (the pull of the wall rows stays in bounds)
     D.plane = (int64_t)D.pitch * (p.ny + (p.walls_y ? 2 : 0));
     const int nchunks = (p.nx + D.V - 1) / D.V;
     D.seg_per_row = (nchunks + 31) / 32;
@@ -278,14 +278,12 @@ void fill_dom(DomDev& D, const lbm_params& p, int kind) {
     D.hot_f.pad = 0.0f;
 }
 
-// Per-node flag words and per-chunk bits (mailbox bounce-back).  Flag bit j
-// (1..8) marks a fluid node whose neighbour x + e_j is solid or lies in a
-// ghost row beyond a y wall (x wrapped when periodic; beyond an open end
-// there is no neighbour); the node writes its f*_j into that neighbour's slot
-// opp(j) after each collision.  On a solid node bit i marks its slot i as such
-// a mailbox (the node x + e_i is fluid); its other slots are read by nobody.  Open columns carry the Zou-He bits, except on
-// wall rows, whose end nodes carry NF_CORNER (their sources beyond the x
-// range reflect from the node's own opposite slot); solid nodes NF_SOLID.  A
+// Per-node flag words and per-chunk bits.  Flag bit j (1..8) marks a fluid node
+// whose neighbour x + e_j is solid or lies beyond a y wall (x wrapped when
+// periodic; beyond an open end there is no neighbour): what it sent there comes
+// back as its population opp(j).  Open columns carry the Zou-He bits, except on
+// wall rows, whose end nodes carry NF_CORNER (their sources beyond the x range
+// reflect from the node's own opposite slot); solid nodes NF_SOLID alone.  A
 // chunk bit is set when any of its nodes has a nonzero flag word.
 void build_flags(const DomDev& D, const uint8_t* solid, std::vector<uint16_t>& fl, std::vector<uint32_t>& words) {
     fl.assign((size_t)D.plane, 0);
@@ -298,21 +296,7 @@ void build_flags(const DomDev& D, const uint8_t* solid, std::vector<uint16_t>& f
             uint16_t f = 0;
             const bool wall_row = wy && (y == 0 || y == D.ny - 1);
             if (solid[(size_t)y * D.nx + x]) {
-                // bit i of a solid node: slot i is a mailbox, i.e. the node
-                // x + e_i exists (wrapped when periodic) and is fluid, and writes it
                 f = NF_SOLID;
-                for (int i = 1; i < 9; ++i) {
-                    int tx = x + ex[i], ty = y + ey[i];
-                    if (ty < 0 || ty >= D.ny) {
-                        if (wy) continue;
-                        ty = (ty + D.ny) % D.ny;
-                    }
-                    if (tx < 0 || tx >= D.nx) {
-                        if (!px) continue;
-                        tx = (tx + D.nx) % D.nx;
-                    }
-                    if (!solid[(size_t)ty * D.nx + tx]) f |= (uint16_t)(1u << i);
-                }
             } else {
                 for (int j = 1; j < 9; ++j) {
                     int tx = x + ex[j], ty = y + ey[j];
@@ -454,8 +438,8 @@ cudaError_t enqueue_stream_collide(lbm_ctx* c, int cur, cudaStream_t s, int bloc
 // launch of forces, exchange and Newton-Euler; the rasterisation and marks
 // for step t+1 and the Eq. MP2 sums for t+2 (they need the state of t+1
 // only); then the stream-collide pass over every item.
-cudaError_t enqueue_step(lbm_ctx* c, int cur, cudaStream_t s) {
-    if (c->np_active == 0) return enqueue_stream_collide(c, cur, s, c->block, c->grid, STREAM_ALL);
+cudaError_t enqueue_step(lbm_ctx* c, int cur, cudaStream_t s, bool pdl) {
+    if (c->np_active == 0) return enqueue_stream_collide(c, cur, s, c->block, c->grid, STREAM_ALL, true, pdl);
     const PartArgs a = part_args(c, cur);
     cudaError_t e;
     if ((e = launch_particle_step(c->kind, a, PL_STEP_A, s)) != cudaSuccess) return e;
@@ -536,7 +520,7 @@ int capture_steps(lbm_ctx* c, int k, int nsteps, cudaGraphExec_t* out) {
     cudaError_t e = cudaSuccess;
     if (c->np_active > 0 && c->overlap) e = enqueue_graph_chains(c, k, nsteps, c->cap_stream);
     else
-        for (int s = 0; s < nsteps && e == cudaSuccess; ++s) e = enqueue_step(c, k ^ (s & 1), c->cap_stream);
+        for (int s = 0; s < nsteps && e == cudaSuccess; ++s) e = enqueue_step(c, k ^ (s & 1), c->cap_stream, s > 0);
     if (e == cudaSuccess && c->np_active > 0 && !c->overlap)
         e = cudaEventRecordWithFlags(c->ev_pstate, c->cap_stream, cudaEventRecordExternal);
     cudaError_t e2 = cudaStreamEndCapture(c->cap_stream, &g);
@@ -815,7 +799,6 @@ int lbm_create_ensemble(int ndom, const lbm_params* per_domain, void* cuda_strea
         if ((r = upload_geometry(c, d)) != LBM_OK) { g_create_error = c->msg; return cleanup(r); }
     // rest state in arena 0
     CKCR(launch_fill_rest(c->kind, c->dd, ndom, c->hd.data(), c->f[0], c->solid, c->stream));
-    for (int d = 0; d < ndom; ++d) CKCR(launch_prime_mail(c->kind, c->hd[d], c->f[0], c->nflags, c->stream));
     if (c->np_slots > 0) {
         c->hst.assign(c->np_slots, PartStatic{});
         for (auto& s : c->hst) s.dom = -1;
@@ -886,7 +869,6 @@ int lbm_set_geometry(lbm_ctx* c, int dom, const uint8_t* solid) {
     if (r) return r;
     CKC(c, launch_export(c->kind, D, c->f[c->cur], c->solid, c->d_stage, c->stream));
     CKC(c, launch_import(c->kind, D, c->d_stage, c->f[c->cur], c->solid, c->stream));
-    CKC(c, launch_prime_mail(c->kind, D, c->f[c->cur], c->nflags, c->stream));
     return sync_and_check(c);
 }
 
@@ -998,7 +980,6 @@ int lbm_set_populations(lbm_ctx* c, int dom, const double* f) {
     if (r) return r;
     CKC(c, cudaMemcpyAsync(c->d_stage, f, bytes, cudaMemcpyHostToDevice, c->stream));
     CKC(c, launch_import(c->kind, D, c->d_stage, c->f[c->cur], c->solid, c->stream));
-    CKC(c, launch_prime_mail(c->kind, D, c->f[c->cur], c->nflags, c->stream));
     return sync_and_check(c);
 }
 

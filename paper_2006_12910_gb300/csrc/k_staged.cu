@@ -86,48 +86,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
     return false;
 }
 
-// A node at x = 0 or nx - 1: sources beyond the x range are read wrapped
-// (periodic x) or patched (Zou-He column, wall-corner reflection).
-template <class S>
-__device__ __noinline__ void seam_node(const DomDev& D, const typename S::T* base, int x, int y, uint32_t fl,
-                                       typename S::A* f) {
-    typedef typename S::A A;
-    const Geo G = load_geo(D);
-    // scaled half-precision stores stay in their scaled units (collide_node<..., SC>)
-    const A inv = S::SCALED ? (A)1 : (A)(sizeof(A) == 4 ? D.inv_scale_f : D.inv_scale);
-    const A sc = S::SCALED ? (A)(sizeof(A) == 4 ? D.scale_f : D.scale) : (A)1;
-    int ym, yp;
-    pull_rows(G, y, ym, yp);
-#pragma unroll
-    for (int i = 1; i < 9; ++i) {
-        const int sx = x - cx(i);
-        if (sx < 0 || sx >= G.nx) {
-            const int row = cy(i) == 1 ? ym : (cy(i) == -1 ? yp : y);
-            if (G.flags & FLAG_PX)
-                f[i] = load_one<S>(base + (int64_t)i * G.plane + (int64_t)row * G.pitch + (sx < 0 ? G.nx - 1 : 0), inv);
-            else if (fl & NF_CORNER)
-                f[i] = load_one<S>(base + (int64_t)opp(i) * G.plane + (int64_t)y * G.pitch + x, inv);
-            else
-                f[i] = (A)0;
-        }
-    }
-    if (fl & NF_ZH_IN) zou_he<A>(f, 0, zou_he_excess<A>(D, 0) * sc);
-    else if (fl & NF_ZH_OUT) zou_he<A>(f, 1, zou_he_excess<A>(D, 1) * sc);
-}
-
-// Mailbox writes of one node (flag bits 1..8), out of line.
-template <class S>
-__device__ __noinline__ void mail_call(const DomDev& D, typename S::T* obase, int x, int y, uint32_t fl,
-                                       const typename S::A* f) {
-    typedef typename S::A A;
-    const Geo G = load_geo(D);
-    A v[9];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) v[i] = f[i];
-    // f is in the store's scaled units when S::SCALED: written without scaling
-    mail_node<S>(G, obase, x, y, fl, v, S::SCALED ? (A)1 : (A)(sizeof(A) == 4 ? D.scale_f : D.scale));
-}
-
 template <class S>
 struct StageGeom {
     typedef typename S::T T;
@@ -156,7 +114,8 @@ __global__ void __launch_bounds__(STAGED_MAX_BLOCK) k_stream_staged(StreamArgs a
     typedef typename S::T T;
     typedef typename S::A A;
     typedef StageGeom<S> SG;
-    constexpr int V = S::V, NW = SG::NW, E = SG::E, ROWE = SG::ROWE;
+    typedef typename ChunkOf<S>::W W;
+    constexpr int V = S::V, NP = ChunkOf<S>::N, NW = SG::NW, E = SG::E, ROWE = SG::ROWE;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
@@ -228,33 +187,43 @@ __global__ void __launch_bounds__(STAGED_MAX_BLOCK) k_stream_staged(StreamArgs a
         const int dn = __shfl_sync(0xffffffffu, c_dn, c);
         const int y = __shfl_sync(0xffffffffu, c_y, c);
         const int sg = __shfl_sync(0xffffffffu, c_seg, c);
+        // Lanes 0-8 copy one plane's row segment each, lanes 9-14 the 16-byte
+        // blocks that hold the wrapped elements of a row end (periodic x: the
+        // last block of the row into the left halo, the first into the right
+        // one), lane 15 the flag words.
+        const Geo G = a.ndom == 1 ? param_geo(a.dom0) : load_geo(a.doms[dn & 0x7fffffff]);
+        const int seg = sg & 0x3fffffff;
+        const int64_t pitch = G.pitch, xs = (int64_t)seg * NW;
+        int ym, yp;
+        pull_rows(G, y, ym, yp);
+        const int64_t w0 = xs >= E ? xs - E : 0;
+        const bool px = G.flags & FLAG_PX, left = px && seg == 0, right = px && xs + NW >= G.nx;
+        const int64_t wr = right ? xs + NW : xs + NW + E;  // a wrapped block fills the right halo
+        const int64_t w1 = wr < pitch ? wr : pitch;
+        const uint32_t bytes = (uint32_t)((w1 - w0) * (int64_t)sizeof(T));
+        const bool spec = (sg >> 30) & 1;
+        const uint32_t fbytes = spec ? (uint32_t)(((xs + NW < pitch ? xs + NW : pitch) - xs) * 2) : 0u;
+        const uint32_t bar = smem_u32(bars + s);
         if (lane == 0) {
-            const Geo G = load_geo(a.doms[dn & 0x7fffffff]);
-            const int64_t pitch = G.pitch;
-            const int seg = sg & 0x3fffffff;
-            const int64_t xs = (int64_t)seg * NW;
-            int ym, yp;
-            pull_rows(G, y, ym, yp);
-            const int64_t w0 = xs >= E ? xs - E : 0;
-            const int64_t w1 = xs + NW + E < pitch ? xs + NW + E : pitch;
-            const uint32_t bytes = (uint32_t)((w1 - w0) * (int64_t)sizeof(T));
-            const bool spec = (sg >> 30) & 1;
-            const int64_t f1 = xs + NW < pitch ? xs + NW : pitch;
-            const uint32_t fbytes = spec ? (uint32_t)((f1 - xs) * 2) : 0u;
             info[s] = make_int4(dn, y, sg, 0);
-            const uint32_t bar = smem_u32(bars + s);
             fence_proxy_async_smem();
-            mbar_arrive_expect_tx(bar, 9u * bytes + fbytes);
-            unsigned char* st = wbuf + (size_t)s * SG::STAGE_B;
-            const uint32_t dst0 = smem_u32(st) + (uint32_t)((w0 - (xs - E)) * (int64_t)sizeof(T));
-            const T* base = src + G.off;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                const int row = cy(i) == 1 ? ym : (cy(i) == -1 ? yp : y);
-                bulk_copy_g2s(dst0 + (uint32_t)(i * ROWE * (int)sizeof(T)), base + i * G.plane + row * pitch + w0,
-                              bytes, bar);
-            }
-            if (spec) bulk_copy_g2s(smem_u32(st + SG::ROWS_B), a.nflags + G.node_off + y * pitch + xs, fbytes, bar);
+            mbar_arrive_expect_tx(bar, 9u * bytes + fbytes + (left ? 48u : 0u) + (right ? 48u : 0u));
+        }
+        __syncwarp();
+        const uint32_t st = smem_u32(wbuf + (size_t)s * SG::STAGE_B);
+        const T* base = src + G.off;
+        if (lane < 15) {
+            // plane and, for the halo blocks, the direction family: +x (1, 5, 8) left, -x (3, 6, 7) right
+            const int i = lane < 9 ? lane : (int)((0x763851u >> (4 * (lane - 9))) & 15u);
+            const int ci = lane < 9 ? 0 : (lane < 12 ? 1 : -1);
+            const int row = (0x64 >> i) & 1 ? ym : ((0x190 >> i) & 1 ? yp : y);  // planes 2, 5, 6 / 4, 7, 8
+            const T* p = base + i * G.plane + row * pitch;
+            const uint32_t d = st + (uint32_t)(i * ROWE * (int)sizeof(T));
+            if (ci == 0) bulk_copy_g2s(d + (uint32_t)((w0 - (xs - E)) * (int64_t)sizeof(T)), p + w0, bytes, bar);
+            else if (ci == 1 && left) bulk_copy_g2s(d, p + (G.nx - 1) / E * E, 16, bar);
+            else if (ci == -1 && right) bulk_copy_g2s(d + (uint32_t)((E + NW) * (int)sizeof(T)), p, 16, bar);
+        } else if (lane == 15 && spec) {
+            bulk_copy_g2s(st + SG::ROWS_B, a.nflags + G.node_off + y * pitch + xs, fbytes, bar);
         }
         __syncwarp();
         return true;
@@ -273,21 +242,15 @@ __global__ void __launch_bounds__(STAGED_MAX_BLOCK) k_stream_staged(StreamArgs a
         const bool near_item = it.x < 0;
         const int y = it.y, seg = it.z & 0x3fffffff;
         const bool spec = (it.z >> 30) & 1;
+        const bool one = a.ndom == 1;
         const DomDev& D = a.doms[d];
-        const Geo G = load_geo(D);
+        const Geo G = one ? param_geo(a.dom0) : load_geo(D);
         const int nx = G.nx;
-        const int64_t pitch = G.pitch, plane = G.plane;
-        const int xs = seg * NW;
+        const int64_t pitch = G.pitch;
         const T* base = src + G.off;
         T* obase = dst + G.off;
-        T* orow = obase + y * pitch + xs;
-        const HotPrm<A> H = load_hot<A>(D);
-        const ExtPrm<A> X = load_ext<A, NOISE, PL>(D);
-        // scaled half-precision stores stay in their scaled units, as in the register kernel
-        const A inv = S::SCALED ? (A)1 : H.inv_scale;
-        const A osc = S::SCALED ? (A)1 : H.scale;
-        int ym, yp;
-        pull_rows(G, y, ym, yp);
+        const HotPrm<A> H = one ? param_hot<A>(a.dom0) : load_hot<A>(D);
+        const ExtPrm<A> X = load_ext<A, NOISE, PL>(one ? a.dom0 : D);
         const bool done = mbar_wait_bounded(smem_u32(bars + sc), (phase >> sc) & 1u, a.wait_ns);
         if (__any_sync(0xffffffffu, !done)) {
             aborted = true;
@@ -298,40 +261,34 @@ __global__ void __launch_bounds__(STAGED_MAX_BLOCK) k_stream_staged(StreamArgs a
 
         const T* sb = reinterpret_cast<const T*>(wbuf + (size_t)sc * SG::STAGE_B);
         const uint16_t* sfl = reinterpret_cast<const uint16_t*>(wbuf + (size_t)sc * SG::STAGE_B + SG::ROWS_B);
-        // Lane l takes nodes xs + l + 32 k: every shared-memory read and every
-        // global store of the warp covers 32 consecutive elements.
-#pragma unroll 2
-        for (int k = 0; k < V; ++k) {
-            const int j = lane + 32 * k;
-            const int x = xs + j;
-            if (x >= nx) continue;
-            const uint32_t fl = spec ? (uint32_t)sfl[j] : 0u;
-            if (fl & NF_SOLID) continue;  // solid slots are mailboxes, written by their fluid neighbours
-            A f[9];
+        const int x0 = seg * NW + lane * V;
+        if (x0 < nx) {
+            const bool px = G.flags & FLAG_PX;
+            // x - 1 of the first node, x + 1 of the last: in the halo, at a
+            // periodic row end in the block that lane 9-14 brought
+            const int jl = x0 == 0 && px ? (nx - 1) % E : E + lane * V - 1;
+            const int jr = x0 + V >= nx && px ? E + NW : E + lane * V + V;
+            Chunk<S> v[9];
+            T e[9];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) f[i] = to_a(sb[i * ROWE + E + j - cx(i)], inv);
-            if (x == 0 || x == nx - 1) {  // rare: through a local copy, so f stays in registers
-                A t[9];
-#pragma unroll
-                for (int i = 0; i < 9; ++i) t[i] = f[i];
-                seam_node<S>(D, base, x, y, fl, t);
-#pragma unroll
-                for (int i = 0; i < 9; ++i) f[i] = t[i];
+            for (int i = 0; i < 9; ++i) {
+                v[i].load_shared(sb + i * ROWE + E + lane * V);
+                if (cx(i)) e[i] = sb[i * ROWE + (cx(i) == 1 ? jl : jr)];
             }
-            ok &= collide_node<A, S::SHIFT, NOISE, PL, S::SCALED>(f, H, X, (uint32_t)(y * nx + x), step);
+            W f[9][NP];
+            form_chunk<S>(v, e, f, nx - 1 - x0);
+            uint16_t fl[V];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) from_a(f[i], osc, orow[(int64_t)i * plane + j]);
-            if (fl & 0x1FEu) {
-                if (mail_is_direct(G, x, y)) {
-                    mail_direct<S>(orow + j, plane, pitch, fl, f, osc);
-                } else {  // rare: wrapped targets, out of line through a local copy
-                    A t[9];
+            for (int k = 0; k < V; ++k) fl[k] = 0;
+            if (spec) {
+                uint32_t any = 0;
 #pragma unroll
-                    for (int i = 0; i < 9; ++i) t[i] = f[i];
-                    mail_call<S>(D, obase, x, y, fl, t);
-                }
+                for (int k = 0; k < V; ++k) any |= fl[k] = sfl[lane * V + k];
+                if (any) patch_chunk<S>(D, G, H.scale, f, fl, y, x0, base);
             }
-            if (FLIPS && near_item) flip_moments<S>(a, D, y, x, obase, next_stamp);
+            ok &= finish_chunk<S, NOISE, PL, FLIPS>(a, D, G, H, X, f, solid_nodes<V>(fl, nx - x0), y, x0, obase,
+                                                    reinterpret_cast<char*>(obase + y * pitch),
+                                                    (uint32_t)x0 * (uint32_t)sizeof(T), step, near_item, next_stamp);
         }
         __syncwarp();
         if (issue(sc)) pending |= 1u << sc;

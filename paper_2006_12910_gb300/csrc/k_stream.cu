@@ -9,17 +9,21 @@
 // item is one (domain, row, warp segment).  For every direction the lane loads
 // the vector of the source row and, for the two x-shifted families, one
 // extra element at the chunk edge (served by L1 from the neighbour lane's
-// sector), then collides in registers and writes 16-byte vectors.
+// sector), then collides in registers -- FP32 kinds two nodes at a time in the
+// packed instructions -- and writes vectors.
 //
-// Halfway bounce-back needs no patching of the pull: solid nodes and the
-// ghost rows beyond y walls hold, in the slot each fluid neighbour pulls, the
-// value that neighbour bounced back (its mailbox write of the previous step).
-// Chunks that hold a solid node, a mailbox writer, an open column or a
-// wall-corner node are flagged in a per-row bitmask; they read their per-node
-// flag words (Zou-He and corner patches, stores that leave solid slots alone,
-// mailbox writes) and otherwise stay on the same vector path.  Only the
-// ragged last chunk of a row whose width is no multiple of V takes a scalar
-// per-node path.
+// The per-node flag words are loaded for every chunk together with the
+// populations, and a chunk with any flag replaces the populations that no
+// fluid node sent (patch_chunk): halfway bounce-back takes the node's own
+// opposite population, so every chunk stores whole vectors and nothing is
+// written outside it.  (Bounced populations written into the solid
+// neighbours' slots instead needed conditional stores per node and plane and a
+// flag look-up before the loads: 765 instructions an item against 596.)  A
+// ragged last chunk treats the padding beyond the row as solid nodes.
+//
+// Bounds: FP32 stores by HBM and L2 (2048x1024 porous geometry, one graph:
+// 27.5 -> 26.5 us a step; 4096x2048 103.6 -> 103.2, 5.9 TB/s); half-precision
+// stores by latency and issue (18.7 -> 14.4 us); noise and tau* by arithmetic.
 #include "stream_node.cuh"
 
 namespace lbmk {
@@ -39,9 +43,13 @@ __global__ void __launch_bounds__(REG_K1_MAX_BLOCK, (k1_min_blocks<S, NOISE, PL>
     asm volatile("griddepcontrol.wait;" ::: "memory");
     typedef typename S::T T;
     typedef typename S::A A;
-    constexpr int V = S::V;
+    typedef typename ChunkOf<S>::W W;
+    constexpr int V = S::V, NP = ChunkOf<S>::N, EB = sizeof(T);
     const int lane = threadIdx.x & 31;
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    // the same for all lanes (a broadcast, so that the compiler knows it)
+    const uint32_t warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
+    const uint32_t wpb = blockDim.x >> 5;
+    const uint32_t nwarps = gridDim.x * wpb;
     const int64_t step64 = *a.ctr_in;
     // every pass writes the (same) counter of the next state, so whichever
     // pass a later kernel waits for has published it
@@ -51,80 +59,73 @@ __global__ void __launch_bounds__(REG_K1_MAX_BLOCK, (k1_min_blocks<S, NOISE, PL>
     const T* __restrict__ src = static_cast<const T*>(a.src);
     T* __restrict__ dst = static_cast<T*>(a.dst);
     bool ok = true;
-    const int lpar = (int)(step64 % 3);
-    const int64_t count = a.mode == STREAM_NEAR ? (int64_t)__ldg(a.near_cnt + lpar) : a.total_items;
+    const uint32_t count = a.mode == STREAM_NEAR ? (uint32_t)__ldg(a.near_cnt + par) : (uint32_t)a.total_items;
     const int32_t next_stamp = (int32_t)(step64 + 1);
+    const int32_t* mark = a.mark + (int64_t)par * a.total_items;
+    const bool one = a.ndom == 1;
 
-    for (int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < count; w += nwarps) {
-        int64_t g = w;
-        int32_t mark = (int32_t)step64;
-        if (a.mode == STREAM_NEAR) g = __ldg(a.near_list + (int64_t)lpar * a.total_items + w);
-        else if (a.mode == STREAM_FAR || FLIPS) mark = __ldg(a.mark + (int64_t)par * a.total_items + w);
-        const bool one = a.ndom == 1;
-        const int d = one ? 0 : find_domain(a.item_off, a.ndom, g);
+    for (uint32_t w = blockIdx.x * wpb + warp; w < count; w += nwarps) {
+        uint32_t g = w;
+        int32_t mk = (int32_t)step64;
+        if (a.mode == STREAM_NEAR)
+            g = __shfl_sync(0xffffffffu, (uint32_t)__ldg(a.near_list + (int64_t)par * a.total_items + w), 0);
+        else if (a.mode == STREAM_FAR || FLIPS) mk = __ldg(mark + w);
+        const int d = one ? 0 : __shfl_sync(0xffffffffu, find_domain(a.item_off, a.ndom, g), 0);
         const DomDev& D = a.doms[d];
         const Geo G = one ? param_geo(a.dom0) : load_geo(D);
         const int nx = G.nx;
         const int64_t pitch = G.pitch, plane = G.plane;
-        const int local = (int)(g - G.item_off);
+        const int local = (int)(g - (uint32_t)G.item_off);
         const int y = item_row(G, local);
         const int seg = local - y * G.spr;
-        const int x0 = (seg * 32 + lane) * V;
-        const uint32_t word = __ldg(a.special + G.mask_off + (int64_t)y * G.spr + seg);
-        const bool near_item = mark == (int32_t)step64;
-        if (a.mode == STREAM_FAR && near_item) continue;
-        if (x0 >= nx) continue;
-        const HotPrm<A> H = one ? param_hot<A>(a.dom0) : load_hot<A>(D);
-        const ExtPrm<A> X = load_ext<A, NOISE, PL>(one ? a.dom0 : D);
         const T* base = src + G.off;
         T* obase = dst + G.off;
-        if (x0 + V > nx) {  // ragged tail chunk
-#pragma unroll 1
-            for (int k = 0; k < V; ++k)
-                if (x0 + k < nx) {
-                    ok &= slow_node<S, NOISE, PL>(D, x0 + k, y, base, obase, a.nflags, step);
-                    if (FLIPS && near_item) flip_moments<S>(a, D, y, x0 + k, obase, next_stamp);
-                }
-            continue;
-        }
-        const bool special = ((word >> lane) & 1u) != 0;
-        uint16_t fl[V];
-#pragma unroll
-        for (int k = 0; k < V; ++k) fl[k] = 0;
-        if (special) load_flags<V>(a.nflags + G.node_off + y * pitch + x0, fl);
-        // scaled half-precision stores stay in their scaled units (see collide_node)
-        const A inv = S::SCALED ? (A)1 : H.inv_scale;
         int ym, yp;
         pull_rows(G, y, ym, yp);
+        const char* rows[3] = {reinterpret_cast<const char*>(base + y * pitch), reinterpret_cast<const char*>(base + ym * pitch),
+                               reinterpret_cast<const char*>(base + yp * pitch)};
         // x-1 / x+V across a seam: wrapped when periodic; at open ends any
-        // in-range element stands in until the Zou-He or corner patch.
+        // in-range element stands in until the Zou-He or corner patch.  Lanes
+        // beyond the row read chunk 0 and store nothing.
+        const int x0 = (seg * 32 + lane) * V;
+        const bool in_row = x0 < nx;
         int xl = x0 - 1, xr = x0 + V;
         if (xl < 0) xl = (G.flags & FLAG_PX) ? nx - 1 : 0;
-        if (xr >= nx) xr = (G.flags & FLAG_PX) ? xr - nx : nx - 1;
-        A f[9][V];
+        if (xr >= nx) xr = (G.flags & FLAG_PX) ? 0 : nx - 1;
+        const uint32_t xo = in_row ? (uint32_t)x0 * EB : 0u, xlo = in_row ? (uint32_t)xl * EB : 0u,
+                       xro = in_row ? (uint32_t)xr * EB : 0u;
+        // The flag words are loaded for every chunk, with the populations: a load
+        // that waits for a bit of the row's mask first costs more than the 2 bytes
+        // a node.
+        uint16_t fl[V];
+        load_flags<V>(a.nflags + G.node_off + y * pitch + (in_row ? x0 : 0), fl);
+        Chunk<S> v[9];
+        T e[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-            const int row = cy(i) == 1 ? ym : (cy(i) == -1 ? yp : y);
-            const T* p = base + (int64_t)i * plane + row * pitch;
-            A v[V];
-            if constexpr (S::SCALED) load_vec_raw<S>(p + x0, v);
-            else load_vec<S>(p + x0, v, inv);
-            if (cx(i) == 0) {
-#pragma unroll
-                for (int k = 0; k < V; ++k) f[i][k] = v[k];
-            } else if (cx(i) == 1) {  // source x-1
-                f[i][0] = load_one<S>(p + xl, inv);
-#pragma unroll
-                for (int k = 1; k < V; ++k) f[i][k] = v[k - 1];
-            } else {  // source x+1
-#pragma unroll
-                for (int k = 0; k < V - 1; ++k) f[i][k] = v[k + 1];
-                f[i][V - 1] = load_one<S>(p + xr, inv);
-            }
+            const char* p = rows[cy(i) == 0 ? 0 : (cy(i) == 1 ? 1 : 2)] + (int64_t)i * plane * EB;
+            v[i].load(p + xo);
+            if (cx(i)) e[i] = __ldg(reinterpret_cast<const T*>(p + (cx(i) == 1 ? xlo : xro)));
         }
-        ok &= finish_chunk<S, NOISE, PL, FLIPS>(a, D, G, H, X, f, special, fl, y, x0, base, obase, step, near_item,
-                                                next_stamp);
+        const HotPrm<A> H = one ? param_hot<A>(a.dom0) : load_hot<A>(D);
+        const ExtPrm<A> X = load_ext<A, NOISE, PL>(one ? a.dom0 : D);
+        const bool near_item = __shfl_sync(0xffffffffu, mk, 0) == (int32_t)step64;
+        if ((a.mode != STREAM_FAR || !near_item) && in_row) {
+            W f[9][NP];
+            form_chunk<S>(v, e, f, nx - 1 - x0);
+            uint32_t any = 0;
+#pragma unroll
+            for (int k = 0; k < V; ++k) any |= fl[k];
+            if (any) patch_chunk<S>(D, G, H.scale, f, fl, y, x0, base);
+            ok &= finish_chunk<S, NOISE, PL, FLIPS>(a, D, G, H, X, f, solid_nodes<V>(fl, nx - x0), y, x0, obase,
+                                                    reinterpret_cast<char*>(obase + y * pitch), xo, step, near_item,
+                                                    next_stamp);
+        }
+        __syncwarp();
     }
+    // The next pass may be placed on the SMs while the last CTAs finish (it
+    // waits for their completion).
+    asm volatile("griddepcontrol.launch_dependents;");
     if (!ok) atomicOr(a.err, ERR_UNSTABLE);
 }
 

@@ -74,9 +74,6 @@ cudaError_t launch_fill_rest(int kind, const DomDev* doms, int ndom, const DomDe
 // offsets wrap on periodic axes; beyond an open end there is no wall).
 cudaError_t launch_lj_wall(const DomDev& D, const uint8_t* solid, const LjEntry* tab, const int32_t* cnt, int dom,
                            double2* out, cudaStream_t s);
-// Mailbox bounce-back slots of one domain from its stored fluid populations
-// (after any write of the populations other than a step).
-cudaError_t launch_prime_mail(int kind, const DomDev& D, void* arena, const uint16_t* nflags, cudaStream_t s);
 // Host-order FP64 f[9][ny][nx] (device buffer) -> stored populations of one domain.
 cudaError_t launch_import(int kind, const DomDev& D, const double* in, void* arena, const uint8_t* solid,
                           cudaStream_t s);

@@ -40,6 +40,51 @@ __host__ __device__ constexpr double inv_sqrt_wk(int k) {
 __host__ __device__ constexpr double noise_coef(int i, int k) { return wgt(i) * mode_vec(k, i) * inv_sqrt_wk(k); }
 
 // ---------------------------------------------------------------------------
+// Arithmetic of the collision on W = double, float or float2 (two nodes at
+// once in the packed FP32 instructions of this architecture).  Every
+// multiply-add is written out, so that a node's result is the same bits
+// whichever kernel, and whichever form, computes it.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ double vadd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double vsub(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double vmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
+// Components of W, and the same value in all of them.
+template <class W> struct Vec;
+template <> struct Vec<double> {
+    typedef double A;
+    static constexpr int N = 1;
+    static __device__ __forceinline__ double all(double x) { return x; }
+    static __device__ __forceinline__ double get(const double& w, int) { return w; }
+    static __device__ __forceinline__ void set(double& w, int, double x) { w = x; }
+};
+template <> struct Vec<float> {
+    typedef float A;
+    static constexpr int N = 1;
+    static __device__ __forceinline__ float all(float x) { return x; }
+    static __device__ __forceinline__ float get(const float& w, int) { return w; }
+    static __device__ __forceinline__ void set(float& w, int, float x) { w = x; }
+};
+template <> struct Vec<float2> {
+    typedef float A;
+    static constexpr int N = 2;
+    static __device__ __forceinline__ float2 all(float x) { return make_float2(x, x); }
+    static __device__ __forceinline__ float get(const float2& w, int k) { return k ? w.y : w.x; }
+    static __device__ __forceinline__ void set(float2& w, int k, float x) {
+        if (k) w.y = x;
+        else w.x = x;
+    }
+};
+
+// ---------------------------------------------------------------------------
 // Population storage kinds.  V = consecutive nodes of one row a lane owns in
 // the register stream-collide kernel (one vector load or store of V*sizeof(T)
 // = 8 or 16 bytes per plane).  MINB / MINB_EXT: CTAs of 128 threads the
@@ -89,8 +134,7 @@ __device__ __forceinline__ void from_a(float v, float, float& o) { o = v; }
 __device__ __forceinline__ void from_a(float v, float s, __half& o) { o = __float2half_rn(v * s); }
 __device__ __forceinline__ void from_a(float v, float s, __nv_bfloat16& o) { o = __float2bfloat16_rn(v * s); }
 
-// Vector load (read-only path) and store of V consecutive elements: one
-// 8- or 16-byte access.
+// Vector load (read-only path) of V consecutive elements: one 8- or 16-byte access.
 template <int B> struct VecOf;
 template <> struct VecOf<8> { typedef uint2 type; };
 template <> struct VecOf<16> { typedef uint4 type; };
@@ -102,26 +146,6 @@ __device__ __forceinline__ void load_vec(const typename S::T* p, typename S::A* 
 #pragma unroll
     for (int k = 0; k < S::V; ++k) out[k] = to_a(r.t[k], inv);
 }
-template <class S>
-__device__ __forceinline__ void store_vec(typename S::T* p, const typename S::A* in, typename S::A scale) {
-    typedef typename VecOf<S::V * sizeof(typename S::T)>::type VT;
-    union { VT u; typename S::T t[S::V]; } r;
-#pragma unroll
-    for (int k = 0; k < S::V; ++k) from_a(in[k], scale, r.t[k]);
-    *reinterpret_cast<VT*>(p) = r.u;
-}
-// The register stream-collide kernel keeps the scaled half-precision stores
-// in their scaled units through the collision (collide_node<..., SC = true>):
-// loads and stores then only convert, two values per instruction where the
-// hardware packs them.
-template <class S>
-__device__ __forceinline__ void load_vec_raw(const typename S::T* p, float* out) {
-    static_assert(S::SCALED && S::V == 4, "raw half-precision loads cover 4-node chunks");
-    union { uint2 u; typename S::T t[4]; } r;
-    r.u = __ldg(reinterpret_cast<const uint2*>(p));
-#pragma unroll
-    for (int k = 0; k < 4; ++k) out[k] = to_a(r.t[k], 1.0f);
-}
 __device__ __forceinline__ uint32_t pack2(float a, float b, __half) {
     const __half2 h = __floats2half2_rn(a, b);
     return *reinterpret_cast<const uint32_t*>(&h);
@@ -130,13 +154,29 @@ __device__ __forceinline__ uint32_t pack2(float a, float b, __nv_bfloat16) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<const uint32_t*>(&h);
 }
+// A chunk as the collision takes it: V / Vec<W>::N vectors W (half-precision
+// kinds in their scaled units), one 8- or 16-byte load (read-only path) or store.
+template <class S> struct ChunkOf { typedef float2 W; static constexpr int N = S::V / 2; };
+template <> struct ChunkOf<StF64> { typedef double W; static constexpr int N = StF64::V; };
 template <class S>
-__device__ __forceinline__ void store_vec_raw(typename S::T* p, const float* in) {
-    static_assert(S::SCALED && S::V == 4, "raw half-precision stores cover 4-node chunks");
-    uint2 u;
-    u.x = pack2(in[0], in[1], typename S::T());
-    u.y = pack2(in[2], in[3], typename S::T());
-    *reinterpret_cast<uint2*>(p) = u;
+struct Chunk {  // as loaded; get() converts
+    typedef typename VecOf<S::V * sizeof(typename S::T)>::type VT;
+    union { VT u; typename S::T t[S::V]; };
+    __device__ __forceinline__ Chunk() {}
+    __device__ __forceinline__ void load(const void* p) { u = __ldg(static_cast<const VT*>(p)); }
+    __device__ __forceinline__ void load_shared(const void* p) { u = *static_cast<const VT*>(p); }
+    __device__ __forceinline__ void get(typename ChunkOf<S>::W (&v)[ChunkOf<S>::N]) const {
+        constexpr int N = Vec<typename ChunkOf<S>::W>::N;
+#pragma unroll
+        for (int k = 0; k < S::V; ++k)
+            Vec<typename ChunkOf<S>::W>::set(v[k / N], k % N, to_a(t[k], (typename S::A)1));
+    }
+};
+template <class S>
+__device__ __forceinline__ void store_chunk(void* p, const typename ChunkOf<S>::W (&v)[ChunkOf<S>::N]) {
+    if constexpr (sizeof(typename S::T) == 8) *static_cast<double2*>(p) = make_double2(v[0], v[1]);
+    else if constexpr (sizeof(typename S::T) == 4) *static_cast<float4*>(p) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+    else *static_cast<uint2*>(p) = make_uint2(pack2(v[0].x, v[0].y, typename S::T()), pack2(v[1].x, v[1].y, typename S::T()));
 }
 template <class S>
 __device__ __forceinline__ typename S::A load_one(const typename S::T* p, typename S::A inv) {
@@ -339,88 +379,125 @@ __device__ __forceinline__ A solve_tau_pl(A Astr, const ExtPrm<A>& P) {
 // whose rounding error stays at the scale of f_i rather than of omega f_i.
 // Returns false when rho is not a positive finite number.
 // ---------------------------------------------------------------------------
-template <typename A, bool SHIFT>
-__device__ __forceinline__ void relax_pair(A& fi, A& fo, A e, A w, A usq, A R, A R3, A B, A om, A omega) {
-    const A q = (A)4.5 * e * e - usq;
+// RND_OM: which product of om f + w h is rounded first (om f, else w h).
+template <class W, bool SHIFT, bool RND_OM>
+__device__ __forceinline__ void relax_pair(W& fi, W& fo, W e, typename Vec<W>::A w, W nusq, W R, W R3, W nR3, W B, W om,
+                                           W nomega) {
+    typedef Vec<W> K;
+    typedef typename K::A A;
+    const W q = vfma(vmul(K::all((A)4.5), e), e, nusq);
+    const W h = vfma(R, q, B);
+    const W hp = vfma(R3, e, h), hm = vfma(nR3, e, h);
     if (SHIFT) {
-        const A h = B + R * q;
-        const A k = R3 * e;
-        fi = om * fi + w * (h + k);
-        fo = om * fo + w * (h - k);
+        fi = RND_OM ? vfma(K::all(w), hp, vmul(om, fi)) : vfma(om, fi, vmul(K::all(w), hp));
+        fo = RND_OM ? vfma(K::all(w), hm, vmul(om, fo)) : vfma(om, fo, vmul(K::all(w), hm));
     } else {  // here R = rho, R3 = 3 rho, B = rho
-        const A h = B + R * q;
-        const A k = R3 * e;
-        fi = fi + omega * (w * (h + k) - fi);
-        fo = fo + omega * (w * (h - k) - fo);
+        fi = vfma(nomega, vfma(K::all(-w), hp, fi), fi);
+        fo = vfma(nomega, vfma(K::all(-w), hm, fo), fo);
     }
+}
+
+// True when rho is a positive finite number (below 1e30), from its bits: the
+// FP64 pipe is the scarce one.
+__device__ __forceinline__ bool rho_ok(float rho) { return __float_as_uint(rho) - 1u < 0x7149F2CAu - 1u; }  // 1e30f
+__device__ __forceinline__ bool rho_ok(double rho) {
+    return (unsigned long long)__double_as_longlong(rho) - 1ull < 0x46293E5939A08CEAull - 1ull;  // 1e30
 }
 
 // SC (shifted stores only): f holds (f - w_i rho0) * s in the store's scaled
 // units, s = H.scale, and so does the result; the moments are unscaled once
-// per node (exact: s is a power of two) instead of every population.
-template <typename A, bool SHIFT, bool NOISE, bool PL, bool SC = false>
-__device__ __forceinline__ bool collide_node(A f[9], const HotPrm<A>& H, const ExtPrm<A>& X, uint32_t node,
-                                             uint32_t step) {
+// per node (exact: s is a power of two) instead of every population.  The
+// components of W are consecutive nodes, the first with index `node`; returns
+// their densities.
+template <class W, bool SHIFT, bool NOISE, bool PL, bool SC = false>
+__device__ __forceinline__ W collide_nodes(W (&f)[9], const HotPrm<typename Vec<W>::A>& H,
+                                           const ExtPrm<typename Vec<W>::A>& X, uint32_t node, uint32_t step) {
     static_assert(!SC || SHIFT, "scaled units are those of the shifted stores");
-    const A a = (f[1] + f[5]) + f[8];  // e_x > 0
-    const A b = (f[3] + f[6]) + f[7];  // e_x < 0
-    const A c = (f[2] + f[5]) + f[6];  // e_y > 0
-    const A d = (f[4] + f[7]) + f[8];  // e_y < 0
-    const A s_ = (f[0] + (f[2] + f[4])) + (a + b);
-    const A jx_ = a - b, jy_ = c - d;
+    typedef Vec<W> K;
+    typedef typename K::A A;
+    const W a = vadd(vadd(f[1], f[5]), f[8]);  // e_x > 0
+    const W b = vadd(vadd(f[3], f[6]), f[7]);  // e_x < 0
+    const W c = vadd(vadd(f[2], f[5]), f[6]);  // e_y > 0
+    const W d = vadd(vadd(f[4], f[7]), f[8]);  // e_y < 0
+    const W s_ = vadd(vadd(f[0], vadd(f[2], f[4])), vadd(a, b));
+    const W jx_ = vsub(a, b), jy_ = vsub(c, d);
     // unscaled moments (SC: one multiply each by the power of two 1/s)
-    const A s = SC ? s_ * H.inv_scale : s_;
-    const A jx = SC ? jx_ * H.inv_scale : jx_, jy = SC ? jy_ * H.inv_scale : jy_;
-    const A rho = SHIFT ? H.rho0 + s : s;
-    const A drho = SHIFT ? s : s - H.rho0;
-    const bool ok = (rho > (A)0) && (rho < (A)1e30);
-    const A irho = rcp_rho<A>(rho);
-    A omega = H.omega, om = H.om, tgx = H.tgx, tgy = H.tgy;
+    const W u1 = K::all(H.inv_scale);
+    const W s = SC ? vmul(s_, u1) : s_;
+    const W jx = SC ? vmul(jx_, u1) : jx_, jy = SC ? vmul(jy_, u1) : jy_;
+    const W rho = SHIFT ? vadd(K::all(H.rho0), s) : s;
+    W irho;
+#pragma unroll
+    for (int k = 0; k < K::N; ++k) K::set(irho, k, rcp_rho<A>(K::get(rho, k)));
+    W omega = K::all(H.omega), om = K::all(H.om), tgx = K::all(H.tgx), tgy = K::all(H.tgy);
     if (PL) {
-        const A u1 = SC ? H.inv_scale : (A)1;  // unscaled second moments
-        const A sxy = ((f[5] + f[7]) - (f[6] + f[8])) * u1;
-        const A iso = SHIFT ? drho * (A)(1.0 / 3.0) : rho * (A)(1.0 / 3.0);
-        const A pxx = (a + b) * u1 - iso - jx * jx * irho;
-        const A pyy = (c + d) * u1 - iso - jy * jy * irho;
-        const A pxy = sxy - jx * jy * irho;
-        const A det = pxy * pxy - pxx * pyy;
-        const A Astr = (A)3 * sqrt(fabs(det)) * irho;
-        const A tau = solve_tau_pl<A>(Astr, X);
-        omega = (A)1 / tau;
-        om = (A)1 - omega;
-        tgx = tau * X.gx;
-        tgy = tau * X.gy;
+        const W drho = SHIFT ? s : vsub(s, K::all(H.rho0));
+        const W iso = SHIFT ? vmul(drho, K::all((A)(1.0 / 3.0))) : vmul(rho, K::all((A)(1.0 / 3.0)));
+        W ab = vadd(a, b), cd = vadd(c, d), sxy = vsub(vadd(f[5], f[7]), vadd(f[6], f[8]));
+        if (SC) { ab = vmul(ab, u1); cd = vmul(cd, u1); sxy = vmul(sxy, u1); }  // unscaled second moments
+        const W njr = vmul(irho, K::all((A)-1));
+        const W pxx = vfma(vmul(jx, jx), njr, vsub(ab, iso));
+        const W pyy = vfma(vmul(jy, jy), njr, vsub(cd, iso));
+        const W pxy = vfma(vmul(jx, jy), njr, sxy);
+        const W det = vsub(vmul(pxy, pxy), vmul(pxx, pyy));
+#pragma unroll
+        for (int k = 0; k < K::N; ++k) {
+            const A Astr = (A)3 * sqrt(fabs(K::get(det, k))) * K::get(irho, k);
+            const A tau = solve_tau_pl<A>(Astr, X);
+            const A w = (A)1 / tau;
+            K::set(omega, k, w);
+            K::set(om, k, (A)1 - w);
+            K::set(tgx, k, tau * X.gx);
+            K::set(tgy, k, tau * X.gy);
+        }
     }
-    const A ux = (jx + rho * tgx) * irho;
-    const A uy = (jy + rho * tgy) * irho;
-    const A usq = (A)1.5 * (ux * ux + uy * uy);
+    const W ux = vmul(vfma(rho, tgx, jx), irho);
+    const W uy = vmul(vfma(rho, tgy, jy), irho);
+    const W nusq = vmul(K::all((A)-1.5), vfma(ux, ux, vmul(uy, uy)));
     // in the units of f (SC: times s)
-    const A R = SHIFT ? (SC ? omega * rho * H.scale : omega * rho) : rho;
-    const A B = SHIFT ? omega * (SC ? s_ : drho) : rho;
-    const A R3 = (A)3 * R;
-    if (SHIFT) f[0] = om * f[0] + (A)wgt(0) * (B - R * usq);
-    else f[0] = f[0] + omega * ((A)wgt(0) * (B - R * usq) - f[0]);
-    relax_pair<A, SHIFT>(f[1], f[3], ux, (A)wgt(1), usq, R, R3, B, om, omega);
-    relax_pair<A, SHIFT>(f[2], f[4], uy, (A)wgt(2), usq, R, R3, B, om, omega);
-    relax_pair<A, SHIFT>(f[5], f[7], ux + uy, (A)wgt(5), usq, R, R3, B, om, omega);
-    relax_pair<A, SHIFT>(f[6], f[8], uy - ux, (A)wgt(6), usq, R, R3, B, om, omega);
+    const W R = SHIFT ? (SC ? vmul(vmul(omega, rho), K::all(H.scale)) : vmul(omega, rho)) : rho;
+    const W B = SHIFT ? vmul(omega, SC ? s_ : s) : rho;
+    const W R3 = vmul(K::all((A)3), R), nR3 = vmul(K::all((A)-3), R);
+    const W nomega = vmul(K::all((A)-1), omega);
+    const W h0 = vfma(R, nusq, B);
+    if (SHIFT) f[0] = vfma(om, f[0], vmul(K::all((A)wgt(0)), h0));
+    else f[0] = vfma(nomega, vfma(K::all(-(A)wgt(0)), h0, f[0]), f[0]);
+    relax_pair<W, SHIFT, false>(f[1], f[3], ux, (A)wgt(1), nusq, R, R3, nR3, B, om, nomega);
+    relax_pair<W, SHIFT, false>(f[2], f[4], uy, (A)wgt(2), nusq, R, R3, nR3, B, om, nomega);
+    relax_pair<W, SHIFT, false>(f[5], f[7], vadd(ux, uy), (A)wgt(5), nusq, R, R3, nR3, B, om, nomega);
+    // (the half-precision stores turn any other rounding into differences of an
+    // ulp of theirs, so the last pair keeps the order it always had)
+    relax_pair<W, SHIFT, !NOISE && !PL>(f[6], f[8], vsub(uy, ux), (A)wgt(6), nusq, R, R3, nR3, B, om, nomega);
     if (NOISE) {
         if (X.kT > (A)0) {
-            A th[6];
-            thetas<A>(node, step, X.dom_id, X.seed, th);
-            const A amp = SC ? sqrt(rho * X.kT * omega * ((A)2 - omega) * (A)3) * H.scale
-                             : sqrt(rho * X.kT * omega * ((A)2 - omega) * (A)3);
+            W th[6], amp;
+#pragma unroll
+            for (int k = 0; k < K::N; ++k) {
+                A t[6];
+                thetas<A>(node + k, step, X.dom_id, X.seed, t);
+#pragma unroll
+                for (int m = 0; m < 6; ++m) K::set(th[m], k, t[m]);
+                const A w = K::get(omega, k);
+                const A am = sqrt(K::get(rho, k) * X.kT * w * ((A)2 - w) * (A)3);
+                K::set(amp, k, SC ? am * H.scale : am);
+            }
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
-                A z = (A)0;
+                W z = K::all((A)0);
 #pragma unroll
                 for (int k = 3; k < 9; ++k)
-                    if (noise_coef(i, k) != 0.0) z += (A)noise_coef(i, k) * th[k - 3];
-                f[i] += amp * z;
+                    if (noise_coef(i, k) != 0.0) z = vfma(K::all((A)noise_coef(i, k)), th[k - 3], z);
+                f[i] = vfma(amp, z, f[i]);
             }
         }
     }
-    return ok;
+    return rho;
+}
+// One node; false when its density is not a positive finite number.
+template <typename A, bool SHIFT, bool NOISE, bool PL, bool SC = false>
+__device__ __forceinline__ bool collide_node(A (&f)[9], const HotPrm<A>& H, const ExtPrm<A>& X, uint32_t node,
+                                             uint32_t step) {
+    return rho_ok(collide_nodes<A, SHIFT, NOISE, PL, SC>(f, H, X, node, step));
 }
 
 // Zou-He density column (Zou & He 1997).  side 0: inlet at x = 0, the

@@ -29,8 +29,8 @@ struct alignas(16) HotPrm {
 // One lattice domain as the kernels see it.  Populations of plane i live at
 // arena[off + i*plane + y*pitch + x]; with y walls each plane also holds one
 // ghost row on each side (y = -1 and y = ny, still addressed as off + i*plane
-// + y*pitch + x), whose slots carry the bounced-back populations of the wall
-// rows.  Per-node solid bytes, flag words and tags at
+// + y*pitch + x), which the wall rows' vector loads read and bounce-back
+// replaces.  Per-node solid bytes, flag words and tags at
 // nodes[node_off + y*pitch + x], 0 <= y < ny; the special-chunk bitmask word of
 // warp segment s of row y at special[mask_off + y*seg_per_row + s] (bit =
 // lane; a chunk is V nodes).
@@ -58,19 +58,11 @@ struct alignas(16) DomDev {
     float n_pl_f, xi_pl_f, tau_min_f, tau_max_f, tmin_pow_f, tmax_pow_f, scale_f, inv_scale_f;
 };
 
-// Per-node flag words (uint16), written from the geometry on the host.
-// Halfway bounce-back uses the slots of solid nodes and wall ghost rows as
-// mailboxes: a fluid node whose neighbour x + e_j is solid or a ghost-row
-// node carries bit j (1..8), and after its collision it writes its outgoing
-// f*_j into slot opp(j) of that neighbour, the slot it pulls direction opp(j)
-// from in the next step.  Pulls therefore need no patching, except at the
-// wall-corner nodes of open ends (NF_CORNER: the directions whose source lies
-// beyond the x range take the node's own opposite slot) and on the Zou-He
-// columns.  On a solid node bits 1..8 mark instead which of its slots are
-// mailboxes (slot i, when the node x + e_i is fluid); no fluid node ever reads
-// the other slots of a solid node, so a chunk may overwrite those with its
-// vector stores.  A chunk whose nodes all have zero flags takes the plain
-// vector path without reading them.
+// Per-node flag words (uint16), written from the geometry on the host.  Bit j
+// (1..8): the neighbour x + e_j of a fluid node is solid or lies beyond a y
+// wall, and the node pulls its population opp(j) from its own slot j instead
+// (halfway bounce-back).  A chunk whose nodes all have zero flags takes the
+// plain vector path without reading them.
 enum : uint16_t {
     NF_SOLID = 1u << 0,
     NF_ZH_IN = 1u << 9,    // Zou-He inlet node (x = 0)

@@ -1,9 +1,8 @@
 // stream_node.cuh -- per-node and per-chunk pieces shared by the two
 // stream-collide kernels (register-pipelined k_stream.cu, staged k_staged.cu):
-// domain geometry loads, the scalar ragged-tail node, flag-word loads,
-// mailbox bounce-back writes, the moments of nodes that change side, and the
-// finish of one pulled V-node chunk (Zou-He and corner patches, collision,
-// stores).  arXiv:2006.12910 Sec. 2 Eqs. e.LB1 /
+// domain geometry loads, flag-word loads, the moments of nodes that change
+// side, and the parts of one V-node chunk (pulled vectors, bounce-back, Zou-He
+// and corner patches, collision, stores).  arXiv:2006.12910 Sec. 2 Eqs. e.LB1 /
 // e.LB2, Sec. 3 (halfway bounce-back, Zou-He), Sec. 4 (noise), Sec. 5 (tau*).
 #pragma once
 #include <cstddef>
@@ -62,7 +61,7 @@ __device__ __forceinline__ int item_row(const Geo& G, int local) {
 }
 
 // Rows that row y pulls from: y -/+ 1, wrapped when periodic in y; with y
-// walls the ghost rows y = -1 and y = ny hold the bounced-back populations.
+// walls y = -1 and y = ny are ghost rows, whose values bounce-back replaces.
 __device__ __forceinline__ void pull_rows(const Geo& G, int y, int& ym, int& yp) {
     ym = y - 1;
     yp = y + 1;
@@ -70,87 +69,6 @@ __device__ __forceinline__ void pull_rows(const Geo& G, int y, int& ym, int& yp)
         if (ym < 0) ym = G.ny - 1;
         if (yp >= G.ny) yp = 0;
     }
-}
-
-// Halfway bounce-back through mailboxes: a fluid node whose neighbour
-// x + e_j is solid or a ghost-row node (flag bit j) writes its post-collision
-// f*_j into slot opp(j) of that neighbour, from which it pulls direction
-// opp(j) in the next step (x wraps when periodic; with open ends no such
-// neighbour lies beyond the x range).
-template <class S>
-__device__ __forceinline__ void mail_node(const Geo& G, typename S::T* obase, int x, int y, uint32_t bits,
-                                          const typename S::A (&f)[9], typename S::A scale) {
-#pragma unroll
-    for (int j = 1; j < 9; ++j) {
-        if (bits & (1u << j)) {
-            int tx = x + cx(j), ty = y + cy(j);
-            if (tx < 0) tx += G.nx;
-            if (tx >= G.nx) tx -= G.nx;
-            if (G.flags & FLAG_PY) {
-                if (ty < 0) ty += G.ny;
-                if (ty >= G.ny) ty -= G.ny;
-            }
-            from_a(f[j], scale, obase[(int64_t)opp(j) * G.plane + (int64_t)ty * G.pitch + tx]);
-        }
-    }
-}
-
-// Mailbox writes of a node whose neighbours need no wrapping (1 <= x <= nx-2,
-// and 1 <= y <= ny-2 when periodic in y): plain offsets from the node's own
-// element p = obase + y*pitch + x.
-template <class S>
-__device__ __forceinline__ void mail_direct(typename S::T* p, int64_t plane, int64_t pitch, uint32_t bits,
-                                            const typename S::A (&f)[9], typename S::A scale) {
-#pragma unroll
-    for (int j = 1; j < 9; ++j)
-        if (bits & (1u << j)) from_a(f[j], scale, p[opp(j) * plane + cy(j) * pitch + cx(j)]);
-}
-
-// True when the mailbox targets of node (x, y) need no wrapping.
-__device__ __forceinline__ bool mail_is_direct(const Geo& G, int x, int y) {
-    return x > 0 && x < G.nx - 1 && (!(G.flags & FLAG_PY) || (y > 0 && y < G.ny - 1));
-}
-
-// Scalar per-node path for the ragged tail: pull (bounced-back populations
-// come from the mailboxes), wall-corner reflection and Zou-He on the open
-// columns, collision, store and mailbox writes.
-template <class S, bool NOISE, bool PL>
-__device__ __noinline__ bool slow_node(const DomDev& D, int x, int y, const typename S::T* __restrict__ base,
-                                       typename S::T* __restrict__ obase, const uint16_t* __restrict__ nflags,
-                                       uint32_t step) {
-    typedef typename S::A A;
-    const Geo G = load_geo(D);
-    const int64_t ni = (int64_t)y * G.pitch + x;
-    const uint32_t fl = __ldg(nflags + G.node_off + ni);
-    if (fl & NF_SOLID) return true;  // solid slots are mailboxes, written by their fluid neighbours
-    const HotPrm<A> H = load_hot<A>(D);
-    const ExtPrm<A> X = load_ext<A, NOISE, PL>(D);
-    // scaled half-precision stores stay in their scaled units (see collide_node)
-    constexpr bool SC = S::SCALED;
-    const A inv = SC ? (A)1 : H.inv_scale, osc = SC ? (A)1 : H.scale;
-    A f[9];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        int sx = x - cx(i), sy = y - cy(i);
-        if ((G.flags & FLAG_PY) && (sy < 0 || sy >= G.ny)) sy = sy < 0 ? sy + G.ny : sy - G.ny;
-        bool own = false, unknown = false;
-        if (sx < 0 || sx >= G.nx) {
-            if (G.flags & FLAG_PX) sx = sx < 0 ? sx + G.nx : sx - G.nx;
-            else if (fl & NF_CORNER) own = true;
-            else unknown = true;  // Zou-He replaces it
-        }
-        if (own) f[i] = load_one<S>(base + (int64_t)opp(i) * G.plane + ni, inv);
-        else if (unknown) f[i] = (A)0;
-        else f[i] = load_one<S>(base + (int64_t)i * G.plane + (int64_t)sy * G.pitch + sx, inv);
-    }
-    const A zsc = SC ? H.scale : (A)1;
-    if (fl & NF_ZH_IN) zou_he<A>(f, 0, zou_he_excess<A>(D, 0) * zsc);
-    else if (fl & NF_ZH_OUT) zou_he<A>(f, 1, zou_he_excess<A>(D, 1) * zsc);
-    const bool ok = collide_node<A, S::SHIFT, NOISE, PL, SC>(f, H, X, (uint32_t)((int64_t)y * G.nx + x), step);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) from_a(f[i], osc, obase[(int64_t)i * G.plane + ni]);
-    if (fl & 0x1FEu) mail_node<S>(G, obase, x, y, fl, f, osc);
-    return ok;
 }
 
 // V per-node flag words of one chunk (V*2 bytes, aligned).
@@ -168,6 +86,54 @@ __device__ __forceinline__ void load_flags(const uint16_t* p, uint16_t (&fl)[V])
 #pragma unroll
         for (int k = 0; k < 4; ++k) { fl[2 * k] = (uint16_t)a[k]; fl[2 * k + 1] = (uint16_t)(a[k] >> 16); }
     }
+}
+
+// The nine pulled populations of a chunk from its row vectors v and the edge
+// elements e (x - 1 of the first node for the directions with e_x = 1, x + 1 of
+// the last one for those with e_x = -1).  last: the index of the row's last
+// node in the chunk; in a ragged last chunk (last < V - 1) that node takes the
+// edge element, and the nodes beyond it are padding, whose values reach nobody.
+template <class S>
+__device__ __forceinline__ void form_chunk(const Chunk<S> (&v)[9], const typename S::T (&e)[9],
+                                           typename ChunkOf<S>::W (&f)[9][ChunkOf<S>::N], int last) {
+    typedef typename S::A A;
+    typedef Vec<typename ChunkOf<S>::W> K;
+    constexpr int V = S::V, N = K::N, NP = ChunkOf<S>::N;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        typename ChunkOf<S>::W u[NP];
+        v[i].get(u);
+        if (cx(i) == 0) {
+#pragma unroll
+            for (int q = 0; q < NP; ++q) f[i][q] = u[q];
+        } else if (cx(i) == 1) {  // source x-1
+            K::set(f[i][0], 0, to_a(e[i], (A)1));
+#pragma unroll
+            for (int k = 1; k < V; ++k) K::set(f[i][k / N], k % N, K::get(u[(k - 1) / N], (k - 1) % N));
+        } else {  // source x+1
+#pragma unroll
+            for (int k = 0; k < V - 1; ++k) K::set(f[i][k / N], k % N, K::get(u[(k + 1) / N], (k + 1) % N));
+            K::set(f[i][NP - 1], N - 1, to_a(e[i], (A)1));
+        }
+    }
+    if (last < V - 1) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i)
+            if (cx(i) == -1) {
+#pragma unroll
+                for (int k = 0; k < V - 1; ++k)
+                    if (k == last) K::set(f[i][k / N], k % N, to_a(e[i], (A)1));
+            }
+    }
+}
+// Bits of a chunk's solid nodes and, in a ragged last chunk (left nodes of the
+// row from its first one on), of the padding beyond the row.
+template <int V>
+__device__ __forceinline__ uint32_t solid_nodes(const uint16_t (&fl)[V], int left) {
+    uint32_t m = left < V ? (((1u << V) - 1u) << left) & ((1u << V) - 1u) : 0u;
+#pragma unroll
+    for (int k = 0; k < V; ++k) m |= (uint32_t)(fl[k] & NF_SOLID) << k;
+    return m;
 }
 
 // Moments of a node that changes side this step (tag stamped step + 1): rho
@@ -194,103 +160,100 @@ __device__ __noinline__ void flip_moments(const StreamArgs& a, const DomDev& D, 
     a.flipmom[3 * (int64_t)slot + 2] = jy;
 }
 
-// Everything after the pull of one V-node chunk.  Special chunks (fl holds
-// their flag words): Zou-He and wall-corner patches on the open columns before
-// the collision, per-node stores that leave solid slots (mailboxes) alone,
-// and the mailbox writes after it.  Then the moments of nodes that change
-// side (near items only).
+// Boundary nodes of a special chunk (fl: its flag words), before the collision:
+// halfway bounce-back (flag bit j: the neighbour x + e_j is solid or beyond a y
+// wall, so the population coming from there, opp(j), is the node's own f*_j),
+// then the wall-corner and Zou-He patches of the open columns.  Straight-line
+// selects: a row of disks puts flagged chunks into most warps, and branches per
+// node and direction cost more than the selects they would skip.
+template <class S>
+__device__ __forceinline__ void patch_chunk(const DomDev& D, const Geo& G, typename S::A scale,
+                                            typename ChunkOf<S>::W (&f)[9][ChunkOf<S>::N], const uint16_t (&fl)[S::V],
+                                            int y, int x0, const typename S::T* base) {
+    typedef typename S::A A;
+    typedef Vec<typename ChunkOf<S>::W> K;
+    constexpr int V = S::V, N = K::N;
+    constexpr bool SC = S::SCALED;
+    const int64_t pitch = G.pitch, plane = G.plane;
+    const typename S::T* own = base + y * pitch + x0;
+    uint32_t any = 0;
+#pragma unroll
+    for (int k = 0; k < V; ++k) any |= (fl[k] & NF_SOLID) ? 0u : fl[k];
+    if (any & 0x1FEu) {
+#pragma unroll
+        for (int j = 1; j < 9; ++j) {
+            if (!(any & (1u << j))) continue;
+            Chunk<S> o;
+            typename ChunkOf<S>::W u[ChunkOf<S>::N];
+            o.load(own + j * plane);
+            o.get(u);
+#pragma unroll
+            for (int k = 0; k < V; ++k)
+                if (fl[k] & (1u << j)) K::set(f[opp(j)][k / N], k % N, K::get(u[k / N], k % N));
+        }
+    }
+    if (any & (NF_ZH_IN | NF_ZH_OUT | NF_CORNER)) {
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+            if (fl[k] & NF_CORNER) {  // sources beyond the x range: the node's own opposite slot
+                const int x = x0 + k;
+#pragma unroll
+                for (int i = 1; i < 9; ++i)
+                    if ((x == 0 && cx(i) == 1) || (x == G.nx - 1 && cx(i) == -1))
+                        K::set(f[i][k / N], k % N, load_one<S>(own + (int64_t)opp(i) * plane + k, (A)1));
+            }
+            if (fl[k] & (NF_ZH_IN | NF_ZH_OUT)) {
+                A n9[9];
+#pragma unroll
+                for (int i = 0; i < 9; ++i) n9[i] = K::get(f[i][k / N], k % N);
+                const int side = (fl[k] & NF_ZH_IN) ? 0 : 1;
+                zou_he<A>(n9, side, SC ? zou_he_excess<A>(D, side) * scale : zou_he_excess<A>(D, side));
+#pragma unroll
+                for (int i = 0; i < 9; ++i) K::set(f[i][k / N], k % N, n9[i]);
+            }
+        }
+    }
+}
+
+// Collision and stores of one chunk, f[i] its pulled populations i as vectors
+// W of the collision (scaled half-precision kinds in their scaled units), solid
+// the bits of its solid and padding nodes: they compute on values that mean
+// nothing, their slots are stored with the vectors and read by nobody, and a
+// chunk of them alone stores nothing.  orow: the store row's start, xo: the
+// chunk's byte offset in it.  Then the moments of nodes that change side (near
+// items only).  False when a density is not a positive finite number.
 template <class S, bool NOISE, bool PL, bool FLIPS>
 __device__ __forceinline__ bool finish_chunk(const StreamArgs& a, const DomDev& D, const Geo& G,
                                              const HotPrm<typename S::A>& H, const ExtPrm<typename S::A>& X,
-                                             typename S::A (&f)[9][S::V], bool special, const uint16_t (&fl)[S::V],
-                                             int y, int x0, const typename S::T* base, typename S::T* obase,
-                                             uint32_t step, bool near_item, int32_t next_stamp) {
-    typedef typename S::A A;
-    constexpr int V = S::V;
-    // scaled half-precision stores: f holds scaled values (see collide_node),
-    // so loads and stores here convert without scaling
-    constexpr bool SC = S::SCALED;
-    const A io_inv = SC ? (A)1 : H.inv_scale, io_scale = SC ? (A)1 : H.scale;
-    const int64_t pitch = G.pitch, plane = G.plane;
-    bool ok = true;
-    // any: OR of the fluid nodes' flags (mailbox writes, open-column patches);
-    // mb_planes: planes in which a solid node of the chunk has a mailbox slot
-    uint32_t solid_bits = 0, any = 0, mb_planes = 0;
-    if (special) {
+                                             typename ChunkOf<S>::W (&f)[9][ChunkOf<S>::N], uint32_t solid, int y, int x0,
+                                             typename S::T* obase, char* orow, uint32_t xo, uint32_t step,
+                                             bool near_item, int32_t next_stamp) {
+    typedef typename ChunkOf<S>::W W;
+    typedef Vec<W> K;
+    constexpr int V = S::V, N = K::N;
+    uint32_t good = solid;
 #pragma unroll
-        for (int k = 0; k < V; ++k) {
-            const bool sol = fl[k] & NF_SOLID;
-            solid_bits |= (uint32_t)sol << k;
-            if (sol) mb_planes |= fl[k];
-            else any |= fl[k];
-        }
-        if (any & (NF_ZH_IN | NF_ZH_OUT | NF_CORNER)) {
+    for (int p = 0; p < ChunkOf<S>::N; ++p) {
+        W n9[9];
 #pragma unroll
-            for (int k = 0; k < V; ++k) {
-                if (fl[k] & NF_CORNER) {  // sources beyond the x range: the node's own opposite slot
-                    const int x = x0 + k;
+        for (int i = 0; i < 9; ++i) n9[i] = f[i][p];
+        const W rho = collide_nodes<W, S::SHIFT, NOISE, PL, S::SCALED>(n9, H, X, (uint32_t)(y * G.nx + x0 + p * N), step);
 #pragma unroll
-                    for (int i = 1; i < 9; ++i)
-                        if ((x == 0 && cx(i) == 1) || (x == G.nx - 1 && cx(i) == -1))
-                            f[i][k] = load_one<S>(base + (int64_t)opp(i) * plane + y * pitch + x, io_inv);
-                }
-                if (fl[k] & (NF_ZH_IN | NF_ZH_OUT)) {
-                    A n9[9];
+        for (int k = 0; k < N; ++k)
+            if (rho_ok(K::get(rho, k))) good |= 1u << (p * N + k);
 #pragma unroll
-                    for (int i = 0; i < 9; ++i) n9[i] = f[i][k];
-                    const int side = (fl[k] & NF_ZH_IN) ? 0 : 1;
-                    zou_he<A>(n9, side, SC ? zou_he_excess<A>(D, side) * H.scale : zou_he_excess<A>(D, side));
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) f[i][k] = n9[i];
-                }
-            }
-        }
+        for (int i = 0; i < 9; ++i) f[i][p] = n9[i];
     }
+    if (solid != (1u << V) - 1u) {
 #pragma unroll
-    for (int k = 0; k < V; ++k) {
-        A n9[9];
-#pragma unroll
-        for (int i = 0; i < 9; ++i) n9[i] = f[i][k];
-        const bool rok = collide_node<A, S::SHIFT, NOISE, PL, SC>(n9, H, X, (uint32_t)(y * G.nx + x0 + k), step);
-        ok &= rok || ((solid_bits >> k) & 1u);  // solid nodes compute on mailbox values and are discarded
-#pragma unroll
-        for (int i = 0; i < 9; ++i) f[i][k] = n9[i];
-    }
-    typename S::T* orow = obase + y * pitch + x0;
-    // A plane in which no solid node of the chunk has a mailbox slot is stored
-    // whole (the solid nodes' slots there are read by nobody); otherwise the
-    // fluid nodes are stored one by one.  A chunk of solid nodes only stores
-    // nothing.
-    if (solid_bits != (1u << V) - 1u) {
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            if (!((mb_planes >> i) & 1u)) {
-                if constexpr (SC) store_vec_raw<S>(orow + (int64_t)i * plane, f[i]);
-                else store_vec<S>(orow + (int64_t)i * plane, f[i], H.scale);
-            } else {
-#pragma unroll
-                for (int k = 0; k < V; ++k)
-                    if (!((solid_bits >> k) & 1u)) from_a(f[i][k], io_scale, orow[(int64_t)i * plane + k]);
-            }
-        }
-    }
-    if (any & 0x1FEu) {
-#pragma unroll
-        for (int k = 0; k < V; ++k) {
-            if ((fl[k] & 0x1FEu) && !(fl[k] & NF_SOLID)) {
-                A n9[9];
-#pragma unroll
-                for (int i = 0; i < 9; ++i) n9[i] = f[i][k];
-                if (mail_is_direct(G, x0 + k, y)) mail_direct<S>(orow + k, plane, pitch, fl[k], n9, io_scale);
-                else mail_node<S>(G, obase, x0 + k, y, fl[k], n9, io_scale);
-            }
-        }
+        for (int i = 0; i < 9; ++i)
+            store_chunk<S>(orow + (int64_t)i * G.plane * (int64_t)sizeof(typename S::T) + xo, f[i]);
     }
     if (FLIPS && near_item) {
 #pragma unroll 1
-        for (int k = 0; k < V; ++k) flip_moments<S>(a, D, y, x0 + k, obase, next_stamp);
+        for (int k = 0; k < V && x0 + k < G.nx; ++k) flip_moments<S>(a, D, y, x0 + k, obase, next_stamp);
     }
-    return ok;
+    return good == (1u << V) - 1u;
 }
 
 }  // namespace lbmk
