@@ -259,6 +259,8 @@ void fill_dom(DomDev& D, const lbm_params& p, int kind) {
     D.drho_in_f = (float)D.drho_in; D.drho_out_f = (float)D.drho_out; D.kT_f = (float)D.kT;
     D.n_pl_f = (float)D.n_pl; D.xi_pl_f = (float)D.xi_pl; D.tau_min_f = (float)D.tau_min;
     D.tau_max_f = (float)D.tau_max; D.tmin_pow_f = (float)D.tmin_pow; D.tmax_pow_f = (float)D.tmax_pow;
+    D.var = 3.0 * D.kT * (p.power_law ? 1.0 : D.inv_tau * (2.0 - D.inv_tau));
+    D.var_f = (float)D.var; D.var_lo_f = (float)(D.var - (double)D.var_f);
     D.scale_f = (float)D.scale; D.inv_scale_f = (float)D.inv_scale;
     D.hot_d.omega = 1.0 / p.tau;
     D.hot_d.om = 1.0 - 1.0 / p.tau;

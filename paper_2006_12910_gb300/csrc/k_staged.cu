@@ -286,9 +286,11 @@ __global__ void __launch_bounds__(STAGED_MAX_BLOCK) k_stream_staged(StreamArgs a
                 for (int k = 0; k < V; ++k) any |= fl[k] = sfl[lane * V + k];
                 if (any) patch_chunk<S>(D, G, H.scale, f, fl, y, x0, base);
             }
-            ok &= finish_chunk<S, NOISE, PL, FLIPS>(a, D, G, H, X, f, solid_nodes<V>(fl, nx - x0), y, x0, obase,
+            W th[NP][6];
+            chunk_thetas<S, NOISE, PL>(X, (uint32_t)(y * nx + x0), step, th);
+            ok &= finish_chunk<S, NOISE, PL, FLIPS>(a, D, G, H, X, f, th, solid_nodes<V>(fl, nx - x0), y, x0, obase,
                                                     reinterpret_cast<char*>(obase + y * pitch),
-                                                    (uint32_t)x0 * (uint32_t)sizeof(T), step, near_item, next_stamp);
+                                                    (uint32_t)x0 * (uint32_t)sizeof(T), near_item, next_stamp);
         }
         __syncwarp();
         if (issue(sc)) pending |= 1u << sc;

@@ -109,6 +109,8 @@ __global__ void __launch_bounds__(REG_K1_MAX_BLOCK, (k1_min_blocks<S, NOISE, PL>
         }
         const HotPrm<A> H = one ? param_hot<A>(a.dom0) : load_hot<A>(D);
         const ExtPrm<A> X = load_ext<A, NOISE, PL>(one ? a.dom0 : D);
+        W th[NP][6];
+        chunk_thetas<S, NOISE, PL>(X, (uint32_t)(y * nx + x0), step, th);
         const bool near_item = __shfl_sync(0xffffffffu, mk, 0) == (int32_t)step64;
         if ((a.mode != STREAM_FAR || !near_item) && in_row) {
             W f[9][NP];
@@ -117,8 +119,8 @@ __global__ void __launch_bounds__(REG_K1_MAX_BLOCK, (k1_min_blocks<S, NOISE, PL>
 #pragma unroll
             for (int k = 0; k < V; ++k) any |= fl[k];
             if (any) patch_chunk<S>(D, G, H.scale, f, fl, y, x0, base);
-            ok &= finish_chunk<S, NOISE, PL, FLIPS>(a, D, G, H, X, f, solid_nodes<V>(fl, nx - x0), y, x0, obase,
-                                                    reinterpret_cast<char*>(obase + y * pitch), xo, step, near_item,
+            ok &= finish_chunk<S, NOISE, PL, FLIPS>(a, D, G, H, X, f, th, solid_nodes<V>(fl, nx - x0), y, x0, obase,
+                                                    reinterpret_cast<char*>(obase + y * pitch), xo, near_item,
                                                     next_stamp);
         }
         __syncwarp();

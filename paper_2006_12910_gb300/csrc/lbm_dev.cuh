@@ -194,25 +194,95 @@ __device__ __forceinline__ float load_one<StBF16S>(const __nv_bfloat16* p, float
 // ---------------------------------------------------------------------------
 // Noise of Sec. 4: counter-based random numbers, uniforms, normal deviates.
 // ---------------------------------------------------------------------------
-// Uniform in (0,1) from the top 23 bits, ((x >> 9) + 1/2) / 2^23; exact in FP32
-// and FP64.  FP32: the 23 bits as the mantissa of a number in [1, 2), minus 1,
-// plus 2^-24 -- both steps exact, so this is the same value with no integer
-// to float conversion.
-__device__ __forceinline__ float uni23f(uint32_t x) {
-    return (__uint_as_float(0x3F800000u | (x >> 9)) - 1.0f) + 5.9604644775390625e-08f;
-}
+// Uniform in (0,1) from the top 23 bits, ((x >> 9) + 1/2) / 2^23, exact in FP64
+// and FP32.  FP32: the 23 bits as the mantissa of a number in [1, 2) (one
+// funnel shift), minus 1, plus 2^-24 -- both steps exact, so this is the same
+// value with no integer to float conversion.
+__device__ __forceinline__ float mant23(uint32_t x) { return __uint_as_float(__funnelshift_r(x, 0x7Fu, 9)); }
 __device__ __forceinline__ double uni23d(uint32_t x) { return ((double)(x >> 9) + 0.5) * 1.1920928955078125e-07; }
 
-// FP32: the angle 2 pi b is taken as pi + 2 pi (b - 1/2) with b - 1/2 exact, so
-// the hardware sine / cosine work inside [-pi, pi] (absolute error about 4e-7,
-// far inside the noise tolerance); the radius keeps the accurate logarithm,
-// whose argument reaches 1 - 2^-24.
-__device__ __forceinline__ void box_muller(float a, float b, float& z0, float& z1) {
-    const float r = sqrtf(-2.0f * logf(a));
-    float s, c;
-    __sincosf(6.28318530717958647692f * (b - 0.5f), &s, &c);
-    z0 = -r * c;
-    z1 = -r * s;
+// Theta_3..Theta_8 of Eq. NP2 for one node: counter (node, step, draw, domain).
+// Philox4x32-10 (Salmon, Moraes, Dror & Shaw, SC'11): ten rounds of two
+// 32x32 -> 64-bit multiplies, key bumped by the Weyl constants between rounds.
+// The two draws of one node (counter words 2 = 0 and 1) run with their rounds
+// interleaved, so that they share the key schedule (and the first round's
+// products, which the compiler finds).
+__device__ __forceinline__ void philox4x32_10_x2(uint4& a, uint4& b, uint32_t k0, uint32_t k1) {
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+        if (r) { k0 += 0x9E3779B9u; k1 += 0xBB67AE85u; }
+        const uint64_t a0 = (uint64_t)a.x * 0xD2511F53u, a1 = (uint64_t)a.z * 0xCD9E8D57u;
+        const uint64_t b0 = (uint64_t)b.x * 0xD2511F53u, b1 = (uint64_t)b.z * 0xCD9E8D57u;
+        a = make_uint4((uint32_t)(a1 >> 32) ^ a.y ^ k0, (uint32_t)a1, (uint32_t)(a0 >> 32) ^ a.w ^ k1, (uint32_t)a0);
+        b = make_uint4((uint32_t)(b1 >> 32) ^ b.y ^ k0, (uint32_t)b1, (uint32_t)(b0 >> 32) ^ b.w ^ k1, (uint32_t)b0);
+    }
+}
+
+// Reciprocal square root by the hardware approximation (FP32, x > 0).
+__device__ __forceinline__ float rsqrt_hw(float x) {
+    float y;
+    asm("rsqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// 2 ln u of the uniform with mantissa bits m in [1, 2) as above: u = 2^e (1 + f)
+// with 1 + f in [sqrt(1/2), sqrt 2), ln(1 + f) = f + f^2 (f p(f) - 1/2), p the
+// degree-7 minimax polynomial of (ln(1 + f) - f + f^2 / 2) / f^3 on that interval
+// with weight f^2 (Remez exchange).  Checked on the CPU for all 2^23 values:
+// relative error of ln u at most 1.37 x 2^-24.  The noise variant is bound by
+// arithmetic: in packed pairs this and the square root below take half the
+// instructions of logf and sqrtf (2048x1024 shifted FP32 with noise: 37.5 ->
+// 29.5 us a step, 1,803 -> 1,230 instructions an item with the packed
+// collision).  Against 64 bits the noise of one node is off by 1.620e-7 of its
+// rms (1.625e-7 with logf and sqrtf), set by the hardware sine and cosine.
+template <class W>
+__device__ __forceinline__ W two_ln_uniform(W m) {
+    typedef Vec<W> K;
+    const W u = vadd(vadd(m, K::all(-1.0f)), K::all(5.9604644775390625e-08f));
+    W r, e;
+#pragma unroll
+    for (int k = 0; k < K::N; ++k) {
+        const uint32_t i = __float_as_uint(K::get(u, k));
+        const uint32_t t = (i + (64u << 23) - 0x3F3504F3u) >> 23;  // e + 64 (0x3F3504F3: sqrt(1/2))
+        K::set(r, k, __uint_as_float(i + ((64u - t) << 23)));
+        K::set(e, k, __uint_as_float(0x4B000000u + t));  // 2^23 + 64 + e
+    }
+    const W f = vadd(r, K::all(-1.0f)), ef = vadd(e, K::all(-8388672.0f));
+    W p = K::all(-0.07859606295824051f);
+    p = vfma(p, f, K::all(0.12881644070148468f));
+    p = vfma(p, f, K::all(-0.13128754496574402f));
+    p = vfma(p, f, K::all(0.14181192219257355f));
+    p = vfma(p, f, K::all(-0.16624553501605988f));
+    p = vfma(p, f, K::all(0.2000228613615036f));
+    p = vfma(p, f, K::all(-0.25000810623168945f));
+    p = vfma(p, f, K::all(0.33333316445350647f));
+    const W l = vfma(ef, K::all(0.693147180559945309f), vfma(vmul(f, f), vfma(p, f, K::all(-0.5f)), f));
+    return vadd(l, l);
+}
+
+// Box-Muller pair of the uniforms a, b given by their mantissas: radius
+// sqrt(-2 ln a) from the reciprocal square root and one Newton step, the angle
+// 2 pi b taken as pi + 2 pi (b - 1/2) with b - 1/2 exact, so the hardware sine /
+// cosine work inside [-pi, pi] (absolute error about 4e-7, far inside the noise
+// tolerance).
+template <class W>
+__device__ __forceinline__ void box_muller(W ma, W mb, W& z0, W& z1) {
+    typedef Vec<W> K;
+    const W nx = two_ln_uniform(ma);  // -x, x = r^2
+    const W ang = vmul(vadd(vadd(mb, K::all(-1.5f)), K::all(5.9604644775390625e-08f)), K::all(6.28318530717958647692f));
+    W y, s, c;
+#pragma unroll
+    for (int k = 0; k < K::N; ++k) {
+        K::set(y, k, rsqrt_hw(-K::get(nx, k)));
+        float sk, ck;
+        __sincosf(K::get(ang, k), &sk, &ck);
+        K::set(s, k, sk);
+        K::set(c, k, ck);
+    }
+    const W q = vmul(nx, y);                                               // -r
+    const W nr = vfma(vfma(q, q, nx), vmul(K::all(0.5f), y), q);
+    z0 = vmul(nr, c);
+    z1 = vmul(nr, s);
 }
 __device__ __forceinline__ void box_muller(double a, double b, double& z0, double& z1) {
     const double r = sqrt(-2.0 * log(a));
@@ -221,36 +291,63 @@ __device__ __forceinline__ void box_muller(double a, double b, double& z0, doubl
     z0 = r * c;
     z1 = r * s;
 }
-template <typename A> __device__ __forceinline__ A uni23(uint32_t x);
-template <> __device__ __forceinline__ float uni23<float>(uint32_t x) { return uni23f(x); }
-template <> __device__ __forceinline__ double uni23<double>(uint32_t x) { return uni23d(x); }
 
-// Theta_3..Theta_8 of Eq. NP2 for one node: counter (node, step, draw, domain).
-// Philox4x32-10 (Salmon, Moraes, Dror & Shaw, SC'11): ten rounds of two
-// 32x32 -> 64-bit multiplies, key bumped by the Weyl constants between rounds.
-// The two draws of one node (counter words 2 = 0 and 1) run with their rounds
-// interleaved, so that they share the key schedule.
-__device__ __forceinline__ void philox4x32_10_x2(uint4& a, uint4& b, uint32_t k0, uint32_t k1) {
+// The six normals of the nodes of W, the first with index `node`.
+template <class W>
+__device__ __forceinline__ void thetas(uint32_t node, uint32_t step, uint32_t dom_id, uint64_t seed, W (&th)[6]) {
+    typedef Vec<W> K;
+    uint4 r0[K::N], r1[K::N];
 #pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        if (r) { k0 += 0x9E3779B9u; k1 += 0xBB67AE85u; }
-        const uint32_t alo0 = 0xD2511F53u * a.x, ahi0 = __umulhi(0xD2511F53u, a.x);
-        const uint32_t alo1 = 0xCD9E8D57u * a.z, ahi1 = __umulhi(0xCD9E8D57u, a.z);
-        const uint32_t blo0 = 0xD2511F53u * b.x, bhi0 = __umulhi(0xD2511F53u, b.x);
-        const uint32_t blo1 = 0xCD9E8D57u * b.z, bhi1 = __umulhi(0xCD9E8D57u, b.z);
-        a = make_uint4(ahi1 ^ a.y ^ k0, alo1, ahi0 ^ a.w ^ k1, alo0);
-        b = make_uint4(bhi1 ^ b.y ^ k0, blo1, bhi0 ^ b.w ^ k1, blo0);
+    for (int k = 0; k < K::N; ++k) {
+        r0[k] = make_uint4(node + k, step, 0u, dom_id);
+        r1[k] = make_uint4(node + k, step, 1u, dom_id);
+        philox4x32_10_x2(r0[k], r1[k], (uint32_t)seed, (uint32_t)(seed >> 32));
+    }
+    if constexpr (sizeof(typename K::A) == 8) {
+        box_muller(uni23d(r0[0].x), uni23d(r0[0].y), th[0], th[1]);
+        box_muller(uni23d(r0[0].z), uni23d(r0[0].w), th[2], th[3]);
+        box_muller(uni23d(r1[0].x), uni23d(r1[0].y), th[4], th[5]);
+    } else {
+        W m[6];
+#pragma unroll
+        for (int k = 0; k < K::N; ++k) {
+            const uint32_t x[6] = {r0[k].x, r0[k].y, r0[k].z, r0[k].w, r1[k].x, r1[k].y};
+#pragma unroll
+            for (int j = 0; j < 6; ++j) K::set(m[j], k, mant23(x[j]));
+        }
+#pragma unroll
+        for (int j = 0; j < 6; j += 2) box_muller(m[j], m[j + 1], th[j], th[j + 1]);
     }
 }
 
-template <typename A>
-__device__ __forceinline__ void thetas(uint32_t node, uint32_t step, uint32_t dom_id, uint64_t seed, A th[6]) {
-    const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-    uint4 r0 = make_uint4(node, step, 0u, dom_id), r1 = make_uint4(node, step, 1u, dom_id);
-    philox4x32_10_x2(r0, r1, k0, k1);
-    box_muller(uni23<A>(r0.x), uni23<A>(r0.y), th[0], th[1]);
-    box_muller(uni23<A>(r0.z), uni23<A>(r0.w), th[2], th[3]);
-    box_muller(uni23<A>(r1.x), uni23<A>(r1.y), th[4], th[5]);
+// Noise of Eq. NP2 added to the populations: f_i += amp omega_i sum_k chi_ki
+// Theta_k, with the sums over the modes that have equal weights on a class of
+// directions taken once (33 operations; 47 written out mode by mode).
+template <class W>
+__device__ __forceinline__ void add_noise(W (&f)[9], W amp, const W (&th)[6]) {
+    typedef Vec<W> K;
+    typedef typename K::A A;
+    static_assert(noise_coef(1, 3) == noise_coef(5, 3) && noise_coef(2, 4) == -noise_coef(1, 4) &&
+                      noise_coef(6, 5) == -noise_coef(5, 5) && noise_coef(2, 8) == noise_coef(1, 8) &&
+                      noise_coef(6, 8) == noise_coef(5, 8) && noise_coef(2, 7) == noise_coef(1, 6) &&
+                      noise_coef(5, 7) == noise_coef(5, 6), "Table 1 weights of the directions of one class");
+    W t[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) t[k] = vmul(amp, th[k]);
+    f[0] = vfma(K::all((A)noise_coef(0, 8)), t[5], vfma(K::all((A)noise_coef(0, 3)), t[0], f[0]));
+    const W s3 = vmul(K::all((A)noise_coef(1, 3)), t[0]);
+    const W ax = vfma(K::all((A)noise_coef(1, 8)), t[5], s3), dg = vfma(K::all((A)noise_coef(5, 8)), t[5], s3);
+    const W p = vfma(K::all((A)noise_coef(1, 4)), t[1], ax), q = vfma(K::all((A)noise_coef(2, 4)), t[1], ax);
+    const W d = vfma(K::all((A)noise_coef(5, 5)), t[2], dg), g = vfma(K::all((A)noise_coef(6, 5)), t[2], dg);
+    f[1] = vadd(f[1], vfma(K::all((A)noise_coef(1, 6)), t[3], p));
+    f[3] = vadd(f[3], vfma(K::all((A)noise_coef(3, 6)), t[3], p));
+    f[2] = vadd(f[2], vfma(K::all((A)noise_coef(2, 7)), t[4], q));
+    f[4] = vadd(f[4], vfma(K::all((A)noise_coef(4, 7)), t[4], q));
+    const W e = vadd(t[3], t[4]), h = vsub(t[3], t[4]);
+    f[5] = vadd(f[5], vfma(K::all((A)noise_coef(5, 6)), e, d));
+    f[7] = vadd(f[7], vfma(K::all((A)noise_coef(7, 6)), e, d));
+    f[8] = vadd(f[8], vfma(K::all((A)noise_coef(8, 6)), h, g));
+    f[6] = vadd(f[6], vfma(K::all((A)noise_coef(6, 6)), h, g));
 }
 
 // ---------------------------------------------------------------------------
@@ -283,7 +380,7 @@ template <> __device__ __forceinline__ HotPrm<double> load_hot<double>(const Dom
 
 template <typename A>
 struct ExtPrm {
-    A gx, gy, kT, xi, n, tmin, tmax, tmin_pow, tmax_pow;
+    A gx, gy, kT, var, var_lo, xi, n, tmin, tmax, tmin_pow, tmax_pow;
     int n_is_one;
     uint32_t dom_id;
     uint64_t seed;
@@ -301,6 +398,8 @@ __device__ __forceinline__ ExtPrm<A> load_ext(const DomDev& D) {
     }
     if (NOISE) {
         X.kT = (A)(f ? D.kT_f : D.kT);
+        X.var = (A)(f ? D.var_f : D.var);  // PL: 3 kT alone
+        X.var_lo = (A)(f ? D.var_lo_f : 0.0);
         X.dom_id = D.domain_id;
         X.seed = D.seed;
     }
@@ -407,11 +506,11 @@ __device__ __forceinline__ bool rho_ok(double rho) {
 // SC (shifted stores only): f holds (f - w_i rho0) * s in the store's scaled
 // units, s = H.scale, and so does the result; the moments are unscaled once
 // per node (exact: s is a power of two) instead of every population.  The
-// components of W are consecutive nodes, the first with index `node`; returns
-// their densities.
+// components of W are nodes, th their normals (NOISE and X.kT > 0: thetas());
+// returns their densities.
 template <class W, bool SHIFT, bool NOISE, bool PL, bool SC = false>
 __device__ __forceinline__ W collide_nodes(W (&f)[9], const HotPrm<typename Vec<W>::A>& H,
-                                           const ExtPrm<typename Vec<W>::A>& X, uint32_t node, uint32_t step) {
+                                           const ExtPrm<typename Vec<W>::A>& X, const W (&th)[6]) {
     static_assert(!SC || SHIFT, "scaled units are those of the shifted stores");
     typedef Vec<W> K;
     typedef typename K::A A;
@@ -470,36 +569,26 @@ __device__ __forceinline__ W collide_nodes(W (&f)[9], const HotPrm<typename Vec<
     relax_pair<W, SHIFT, !NOISE && !PL>(f[6], f[8], vsub(uy, ux), (A)wgt(6), nusq, R, R3, nR3, B, om, nomega);
     if (NOISE) {
         if (X.kT > (A)0) {
-            W th[6], amp;
+            W amp;
+            // var = 3 kT omega (2 - omega), as a pair hi + lo where omega is a constant
+            W x;
+            if (PL) x = vmul(rho, vmul(vmul(omega, vsub(K::all((A)2), omega)), K::all(X.var)));
+            else x = vfma(rho, K::all(X.var), vmul(rho, K::all(X.var_lo)));
+            if constexpr (sizeof(A) == 8) {
+                amp = sqrt(x);
+            } else {
+                W y;  // 1 / sqrt(x), 0 where x is not positive (no noise there)
 #pragma unroll
-            for (int k = 0; k < K::N; ++k) {
-                A t[6];
-                thetas<A>(node + k, step, X.dom_id, X.seed, t);
-#pragma unroll
-                for (int m = 0; m < 6; ++m) K::set(th[m], k, t[m]);
-                const A w = K::get(omega, k);
-                const A am = sqrt(K::get(rho, k) * X.kT * w * ((A)2 - w) * (A)3);
-                K::set(amp, k, SC ? am * H.scale : am);
+                for (int k = 0; k < K::N; ++k) K::set(y, k, K::get(x, k) > 0.0f ? rsqrt_hw(K::get(x, k)) : 0.0f);
+                const W r = vmul(x, y);
+                amp = vfma(vfma(vmul(K::all((A)-1), r), r, x), vmul(K::all((A)0.5), y), r);
             }
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                W z = K::all((A)0);
-#pragma unroll
-                for (int k = 3; k < 9; ++k)
-                    if (noise_coef(i, k) != 0.0) z = vfma(K::all((A)noise_coef(i, k)), th[k - 3], z);
-                f[i] = vfma(amp, z, f[i]);
-            }
+            if (SC) amp = vmul(amp, K::all(H.scale));
+            add_noise(f, amp, th);
         }
     }
     return rho;
 }
-// One node; false when its density is not a positive finite number.
-template <typename A, bool SHIFT, bool NOISE, bool PL, bool SC = false>
-__device__ __forceinline__ bool collide_node(A (&f)[9], const HotPrm<A>& H, const ExtPrm<A>& X, uint32_t node,
-                                             uint32_t step) {
-    return rho_ok(collide_nodes<A, SHIFT, NOISE, PL, SC>(f, H, X, node, step));
-}
-
 // Zou-He density column (Zou & He 1997).  side 0: inlet at x = 0, the
 // populations 1, 5, 8 enter from outside; side 1: outlet at x = nx-1, the
 // populations 3, 6, 7 enter.  d_b is the prescribed density in the units of

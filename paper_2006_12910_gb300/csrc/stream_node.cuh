@@ -215,8 +215,28 @@ __device__ __forceinline__ void patch_chunk(const DomDev& D, const Geo& G, typen
     }
 }
 
+// Normals of a chunk's nodes.  They need no population, so the kernels draw them
+// while the loads are in flight.
+template <class S, bool NOISE, bool PL>
+__device__ __forceinline__ void chunk_thetas(const ExtPrm<typename S::A>& X, uint32_t node, uint32_t step,
+                                             typename ChunkOf<S>::W (&th)[ChunkOf<S>::N][6]) {
+    typedef Vec<typename ChunkOf<S>::W> K;
+    if (NOISE) {
+        if (X.kT > (typename S::A)0) {
+#pragma unroll
+            for (int p = 0; p < ChunkOf<S>::N; ++p) thetas(node + p * K::N, step, X.dom_id, X.seed, th[p]);
+            return;
+        }
+    }
+#pragma unroll
+    for (int p = 0; p < ChunkOf<S>::N; ++p)
+#pragma unroll
+        for (int m = 0; m < 6; ++m) th[p][m] = K::all(0);
+}
+
 // Collision and stores of one chunk, f[i] its pulled populations i as vectors
-// W of the collision (scaled half-precision kinds in their scaled units), solid
+// W of the collision (scaled half-precision kinds in their scaled units), th
+// the normals of its nodes, solid
 // the bits of its solid and padding nodes: they compute on values that mean
 // nothing, their slots are stored with the vectors and read by nobody, and a
 // chunk of them alone stores nothing.  orow: the store row's start, xo: the
@@ -225,9 +245,10 @@ __device__ __forceinline__ void patch_chunk(const DomDev& D, const Geo& G, typen
 template <class S, bool NOISE, bool PL, bool FLIPS>
 __device__ __forceinline__ bool finish_chunk(const StreamArgs& a, const DomDev& D, const Geo& G,
                                              const HotPrm<typename S::A>& H, const ExtPrm<typename S::A>& X,
-                                             typename ChunkOf<S>::W (&f)[9][ChunkOf<S>::N], uint32_t solid, int y, int x0,
-                                             typename S::T* obase, char* orow, uint32_t xo, uint32_t step,
-                                             bool near_item, int32_t next_stamp) {
+                                             typename ChunkOf<S>::W (&f)[9][ChunkOf<S>::N],
+                                             const typename ChunkOf<S>::W (&th)[ChunkOf<S>::N][6], uint32_t solid, int y,
+                                             int x0, typename S::T* obase, char* orow, uint32_t xo, bool near_item,
+                                             int32_t next_stamp) {
     typedef typename ChunkOf<S>::W W;
     typedef Vec<W> K;
     constexpr int V = S::V, N = K::N;
@@ -237,7 +258,7 @@ __device__ __forceinline__ bool finish_chunk(const StreamArgs& a, const DomDev& 
         W n9[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) n9[i] = f[i][p];
-        const W rho = collide_nodes<W, S::SHIFT, NOISE, PL, S::SCALED>(n9, H, X, (uint32_t)(y * G.nx + x0 + p * N), step);
+        const W rho = collide_nodes<W, S::SHIFT, NOISE, PL, S::SCALED>(n9, H, X, th[p]);
 #pragma unroll
         for (int k = 0; k < N; ++k)
             if (rho_ok(K::get(rho, k))) good |= 1u << (p * N + k);
