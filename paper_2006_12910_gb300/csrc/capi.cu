@@ -32,6 +32,7 @@ namespace {
 // one graph per binary digit of n mod 2^GRAPH_LOG plus n >> GRAPH_LOG of the
 // largest.
 constexpr int GRAPH_LOG = 6;
+constexpr int64_t SPLIT_ITEMS = 3072;  // see enqueue_graph_chains
 thread_local std::string g_create_error = "no error";
 
 // Test hook of lbm_debug_fail_alloc: when positive, the device allocation
@@ -110,6 +111,7 @@ struct lbm_ctx {
     double* ljf = nullptr;               // [2][np_slots][4]: Eq. MP2 force and torque, copy by step parity
     double* flipmom = nullptr;           // [2][flips_total][3]
     int64_t near_grid = 1;
+    bool any_lj = false;                 // some domain has an Eq. MP2 force
     LjEntry* lj_tab = nullptr;           // [ndom][LJ_TAB]
     double2* ljwall = nullptr;           // per node: Eq. MP2 force from walls / solids (domains with psi > 0)
     int32_t* lj_cnt = nullptr;           // [ndom]
@@ -445,73 +447,103 @@ cudaError_t enqueue_step(lbm_ctx* c, int cur, cudaStream_t s, bool pdl) {
     const PartArgs a = part_args(c, cur);
     cudaError_t e;
     if ((e = launch_particle_step(c->kind, a, PL_STEP_A, s)) != cudaSuccess) return e;
-    if ((e = launch_particle_step(c->kind, a, PL_STEP_R, s)) != cudaSuccess) return e;
-    if ((e = launch_particle_step(c->kind, a, PL_STEP_LJ, s)) != cudaSuccess) return e;
+    if ((e = launch_particle_step(c->kind, a, c->any_lj ? PL_STEP_RLJ : PL_STEP_R, s)) != cudaSuccess) return e;
     return enqueue_stream_collide(c, cur, s, c->block, c->grid, STREAM_ALL);
 }
 
-// nsteps steps with particles, as four chains.  Main stream: the particle
-// launch of forces, exchange and Newton-Euler, and the NEAR pass of every
-// step.  Far stream: the FAR passes.  Raster stream: the rasterisation and
-// near-item marks for the following step, which need only the state that the
-// force launch wrote and so run beside the NEAR pass.  LJ stream: the Eq. MP2
-// sums two steps ahead.  Edges:
+// nsteps steps with particles, as chains of launches.  Main stream: the
+// particle launch of forces, exchange and Newton-Euler, then the stream-collide
+// pass of the step.  Raster stream: the rasterisation and near-item marks for
+// the following step and the Eq. MP2 sums for the one after it, which need only
+// the state that the force launch wrote and so run beside the pass.
+//
+// On lattices of more than SPLIT_ITEMS work items the pass is split: a far
+// stream runs the FAR passes, the main stream the NEAR passes, so that the
+// force launches overlap the bulk of the lattice, and the Eq. MP2 sums (where
+// any domain has them) run on a stream of their own: beside a FAR pass their
+// CTAs would hold back the rasterisation (merged: 831 us a call of 20 steps of
+// the porous workload, 760 apart).  Below, one pass over every item after the
+// force launch ends as early as the near items alone would, and two chains
+// instead of four leave room for other contexts: the device has eight hardware
+// queues by default, and three contexts with four chains each waited for one
+// another (512x512 fluctuating box, calls of 20 steps of three contexts in
+// turn: 201 -> 146 us a call, one context alone 379 -> 386; 3000x41 channel 188
+// -> 131 and 372 -> 368).  SPLIT_ITEMS lies where the whole pass stops being the
+// shorter one (us a step, one context alone, whole / split: 512x512 noise,
+// 2,048 items, 18.0 / 18.2; 820x510 grains, 3,570 items, 21.3 / 23.6; 768x768
+// noise, 4,608 items, 22.4 / 18.8; 1300x820 grains, 9,020 items, 31.8 / 27.5).
+//
+// Edges:
 //  - FAR(t) after NEAR(t-1): the near items of t-1 are the only ones it may
 //    read that the far chain did not write itself;
 //  - NEAR(t) after FAR(t-1) (it overwrites the arena FAR(t-1) read and reads
-//    its output at the seams) and after launch 2 for t (the node tags of
-//    side changes of t);
-//  - the rasterisation for t+1 after the force launch of t (state of t+1; the
-//    lists of t it replaces are read) and after FAR(t-1) (the marks it writes
-//    are the three-way copy FAR(t-1) read);
+//    its output at the seams);
+//  - the pass of t (NEAR or whole) after the raster launch of t-1 (the node
+//    tags of side changes of t);
+//  - the raster launch of t after the force launch of t (state of t+1; the
+//    lists of t it replaces are read) and, when split, after FAR(t-1) (the
+//    marks it writes are the three-way copy FAR(t-1) read);
 //  - the Eq. MP2 sums for t+2 after the force launch of t (state of t+1; the
-//    sums of t they replace are read), and the force launch of t+2 after them.
+//    sums of t they replace are read), and the force launch of t+2 after them
+//    (through the pass of t+1 when they are part of the raster launch).
 // The force launch of t+1 needs nothing from FAR(t): it reads and writes
 // only slots of items near the particles, which NEAR(t) produced.  What the
 // first steps of the graph need from launches of earlier steps ran before it
-// (previous graph or set-up).  Each NEAR pass is a programmatic dependent of
-// the force launch before it: the force launch signals once the particle
-// states are solved, the NEAR CTAs are then placed while its exchange
-// completes and wait for its completion (and for the edges from the other
-// streams) before they touch memory, which takes the launch latency off the
-// particle chain.  (The same for the FAR passes and the force launches
+// (previous graph or set-up).  Each pass on the main stream is a programmatic
+// dependent of the force launch before it: the force launch signals once the
+// particle states are solved, the CTAs of the pass are then placed while its
+// exchange completes and wait for its completion (and for the edges from the
+// other streams) before they touch memory, which takes the launch latency off
+// the particle chain.  (The same for the FAR passes and the force launches
 // measured no faster.)
 cudaError_t enqueue_graph_chains(lbm_ctx* c, int k, int nsteps, cudaStream_t s) {
     cudaError_t e;
+    const bool split = c->total_items > SPLIT_ITEMS, lj_apart = split && c->any_lj;
     if ((e = cudaEventRecord(c->ev_fork, s)) != cudaSuccess) return e;
-    if ((e = cudaStreamWaitEvent(c->far_stream, c->ev_fork, 0)) != cudaSuccess) return e;
+    if (split && (e = cudaStreamWaitEvent(c->far_stream, c->ev_fork, 0)) != cudaSuccess) return e;
+    if (lj_apart && (e = cudaStreamWaitEvent(c->lj_stream, c->ev_fork, 0)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(c->rast_stream, c->ev_fork, 0)) != cudaSuccess) return e;
-    if ((e = cudaStreamWaitEvent(c->lj_stream, c->ev_fork, 0)) != cudaSuccess) return e;
     for (int st = 0; st < nsteps; ++st) {
         const int cur = k ^ (st & 1);
         const PartArgs a = part_args(c, cur);
-        if (st > 0 && (e = cudaStreamWaitEvent(c->far_stream, c->ev_near[(st - 1) & 1], 0)) != cudaSuccess) return e;
-        if ((e = enqueue_stream_collide(c, cur, c->far_stream, c->block, c->grid, STREAM_FAR)) != cudaSuccess) return e;
-        if ((e = cudaEventRecord(c->ev_far[st & 1], c->far_stream)) != cudaSuccess) return e;
-        if (st > 1 && (e = cudaStreamWaitEvent(s, c->ev_lj[st & 1], 0)) != cudaSuccess) return e;  // sums of st
+        if (split) {
+            if (st > 0 && (e = cudaStreamWaitEvent(c->far_stream, c->ev_near[(st - 1) & 1], 0)) != cudaSuccess) return e;
+            if ((e = enqueue_stream_collide(c, cur, c->far_stream, c->block, c->grid, STREAM_FAR)) != cudaSuccess) return e;
+            if ((e = cudaEventRecord(c->ev_far[st & 1], c->far_stream)) != cudaSuccess) return e;
+        }
+        if (lj_apart && st > 1 && (e = cudaStreamWaitEvent(s, c->ev_lj[st & 1], 0)) != cudaSuccess) return e;  // sums of st
         if ((e = launch_particle_step(c->kind, a, PL_STEP_A, s)) != cudaSuccess) return e;
         if (st == nsteps - 1 && (e = cudaEventRecordWithFlags(c->ev_pstate, s, cudaEventRecordExternal)) != cudaSuccess)
             return e;
         if ((e = cudaEventRecord(c->ev_a[st & 1], s)) != cudaSuccess) return e;
-        if ((e = cudaStreamWaitEvent(c->lj_stream, c->ev_a[st & 1], 0)) != cudaSuccess) return e;
-        if ((e = launch_particle_step(c->kind, a, PL_STEP_LJ, c->lj_stream)) != cudaSuccess) return e;
-        if ((e = cudaEventRecord(c->ev_lj[st & 1], c->lj_stream)) != cudaSuccess) return e;
+        if (lj_apart) {
+            if ((e = cudaStreamWaitEvent(c->lj_stream, c->ev_a[st & 1], 0)) != cudaSuccess) return e;
+            if ((e = launch_particle_step(c->kind, a, PL_STEP_LJ, c->lj_stream)) != cudaSuccess) return e;
+            if ((e = cudaEventRecord(c->ev_lj[st & 1], c->lj_stream)) != cudaSuccess) return e;
+        }
         if ((e = cudaStreamWaitEvent(c->rast_stream, c->ev_a[st & 1], 0)) != cudaSuccess) return e;
-        if (st > 0 && (e = cudaStreamWaitEvent(c->rast_stream, c->ev_far[(st - 1) & 1], 0)) != cudaSuccess) return e;
-        if ((e = launch_particle_step(c->kind, a, PL_STEP_R, c->rast_stream)) != cudaSuccess) return e;
+        if (split && st > 0 && (e = cudaStreamWaitEvent(c->rast_stream, c->ev_far[(st - 1) & 1], 0)) != cudaSuccess) return e;
+        e = launch_particle_step(c->kind, a, c->any_lj && !lj_apart ? PL_STEP_RLJ : PL_STEP_R, c->rast_stream);
+        if (e != cudaSuccess) return e;
         if ((e = cudaEventRecord(c->ev_rast[st & 1], c->rast_stream)) != cudaSuccess) return e;
         if (st > 0 && (e = cudaStreamWaitEvent(s, c->ev_rast[(st - 1) & 1], 0)) != cudaSuccess) return e;
-        if (st > 0 && (e = cudaStreamWaitEvent(s, c->ev_far[(st - 1) & 1], 0)) != cudaSuccess) return e;
-        if ((e = enqueue_stream_collide(c, cur, s, near_block(c), c->near_grid, STREAM_NEAR, true, true)) != cudaSuccess)
-            return e;
-        if ((e = cudaEventRecord(c->ev_near[st & 1], s)) != cudaSuccess) return e;
+        if (split) {
+            if (st > 0 && (e = cudaStreamWaitEvent(s, c->ev_far[(st - 1) & 1], 0)) != cudaSuccess) return e;
+            e = enqueue_stream_collide(c, cur, s, near_block(c), c->near_grid, STREAM_NEAR, true, true);
+        } else {
+            e = enqueue_stream_collide(c, cur, s, c->block, c->grid, STREAM_ALL, true, true);
+        }
+        if (e != cudaSuccess) return e;
+        if (split && (e = cudaEventRecord(c->ev_near[st & 1], s)) != cudaSuccess) return e;
     }
-    if ((e = cudaEventRecord(c->ev_join, c->far_stream)) != cudaSuccess) return e;
+    if (split && (e = cudaEventRecord(c->ev_join, c->far_stream)) != cudaSuccess) return e;
     if ((e = cudaEventRecord(c->ev_join2, c->rast_stream)) != cudaSuccess) return e;
-    if ((e = cudaEventRecord(c->ev_join3, c->lj_stream)) != cudaSuccess) return e;
-    if ((e = cudaStreamWaitEvent(s, c->ev_join, 0)) != cudaSuccess) return e;
-    if ((e = cudaStreamWaitEvent(s, c->ev_join2, 0)) != cudaSuccess) return e;
-    return cudaStreamWaitEvent(s, c->ev_join3, 0);
+    if (split && (e = cudaStreamWaitEvent(s, c->ev_join, 0)) != cudaSuccess) return e;
+    if (lj_apart) {
+        if ((e = cudaEventRecord(c->ev_join3, c->lj_stream)) != cudaSuccess) return e;
+        if ((e = cudaStreamWaitEvent(s, c->ev_join3, 0)) != cudaSuccess) return e;
+    }
+    return cudaStreamWaitEvent(s, c->ev_join2, 0);
 }
 
 // Captures nsteps steps starting from state k into one executable graph.
@@ -774,9 +806,8 @@ int lbm_create_ensemble(int ndom, const lbm_params* per_domain, void* cuda_strea
     CKCR(dev_malloc(&c->nflags, c->node_bytes * 2));
     CKCR(dev_malloc(&c->special, std::max<size_t>(1, c->special_words) * 4));
     {
-        bool any_lj = false;
-        for (int d = 0; d < ndom; ++d) any_lj |= per_domain[d].lj_psi > 0.0 && per_domain[d].lj_rit > 0.0;
-        if (any_lj) {
+        for (int d = 0; d < ndom; ++d) c->any_lj |= per_domain[d].lj_psi > 0.0 && per_domain[d].lj_rit > 0.0;
+        if (c->any_lj) {
             CKCR(dev_malloc(&c->ljwall, sizeof(double2) * std::max<size_t>(1, c->node_bytes)));
             CKCR(cudaMemsetAsync(c->ljwall, 0, sizeof(double2) * std::max<size_t>(1, c->node_bytes), c->stream));
         }
@@ -1383,10 +1414,10 @@ int lbm_profile_steps(lbm_ctx* c, int64_t nsteps, double* ms_out3, int64_t* laun
                 if (ce == cudaSuccess) ce = cudaEventRecord(e[0], c->stream);
                 if (ce == cudaSuccess) ce = launch_particle_step(c->kind, a, PL_STEP_A, c->stream);
                 if (ce == cudaSuccess) ce = cudaEventRecord(e[1], c->stream);
-                if (ce == cudaSuccess) ce = launch_particle_step(c->kind, a, PL_STEP_R, c->stream);
-                if (ce == cudaSuccess) ce = launch_particle_step(c->kind, a, PL_STEP_LJ, c->stream);
+                if (ce == cudaSuccess)
+                    ce = launch_particle_step(c->kind, a, c->any_lj ? PL_STEP_RLJ : PL_STEP_R, c->stream);
                 if (ce == cudaSuccess) ce = cudaEventRecord(e[4], c->stream);
-                launches += 3;
+                launches += 2;
             }
             if (ce == cudaSuccess) ce = cudaEventRecord(e[2], c->stream);
             if (ce == cudaSuccess) ce = enqueue_stream_collide(c, c->cur, c->stream, c->block, c->grid);

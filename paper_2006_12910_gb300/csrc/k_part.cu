@@ -1353,9 +1353,10 @@ cudaError_t launch_particle_step(int kind, const PartArgs& a, int modes, cudaStr
     // role A alone uses warps 0-4 only (links, covered / uncovered nodes): a
     // smaller CTA finds room sooner beside a running stream-collide pass
     const int block = r1 == 0 ? A_BLOCK : (r0 >= 2 ? BC_BLOCK : PBLOCK);
-    cudaError_t e = cudaErrorInvalidValue;  // role A or D together with other roles: no such launch
+    cudaError_t e = cudaErrorInvalidValue;  // role A together with other roles: no such launch
     if (r1 == 0) LBM_PDISPATCH(kind, (e = launch_part<S, 0, 0>(a, modes, r0, grid, block, s, pdl)))
     else if (r0 == 1 && r1 == 1) LBM_PDISPATCH(kind, (e = launch_part<S, 1, 1>(a, modes, r0, grid, block, s, pdl)))
+    else if (r0 == 1) LBM_PDISPATCH(kind, (e = launch_part<S, 1, 3>(a, modes, r0, grid, block, s, pdl)))
     else if (r0 >= 2) LBM_PDISPATCH(kind, (e = launch_part<S, 2, 3>(a, modes, r0, grid, block, s, pdl)))
     return e;
 }

@@ -138,11 +138,12 @@ struct PartArgs {
 // the Eq. MP2 sum, and "ahead" (the step is one past the published counter).
 enum { PL_FORCES = 1, PL_SWAP = 2, PL_ADVANCE = 4, PL_RASTER = 8, PL_MARK = 16, PL_LJ = 32, PL_AHEAD = 64 };
 // Launches of step t: forces, exchange and Newton-Euler (role A); after it,
-// the rasterisation and marks for step t+1 (roles B, C) and the Eq. MP2 sum
-// for step t+2 (role D), each on its own stream.
+// the rasterisation and marks for step t+1 (roles B, C) and, where some domain
+// has that force, the Eq. MP2 sum for step t+2 (role D).
 constexpr int PL_STEP_A = PL_FORCES | PL_SWAP | PL_ADVANCE;
 constexpr int PL_STEP_R = PL_RASTER | PL_MARK | PL_ADVANCE | PL_AHEAD;
 constexpr int PL_STEP_LJ = PL_LJ | PL_ADVANCE | PL_AHEAD;
+constexpr int PL_STEP_RLJ = PL_STEP_R | PL_STEP_LJ;
 // set-up at the current step t: rasterisation and marks of t, then PL_SETUP_R
 // (rasterisation and marks of t+1), PL_LJ (Eq. MP2 at t) and
 // PL_LJ | PL_ADVANCE (Eq. MP2 at t+1)
