@@ -52,8 +52,9 @@ extern "C" {
 #define LBM_E_STATE (-6)    /* call order, particle overlap or list capacity */
 #define LBM_E_IO (-7)       /* checkpoint file error */
 
-/* Population storage.  F64 stores f and computes in FP64 (the plain FP64
- * path).  Every other kind computes in FP32 registers: F32 stores f, the
+/* Population storage.  F64 stores f in FP64 and collides in 64-bit arithmetic
+ * (BGK: fixed point in units of 2^-60 or finer of rho0, FP64 for nodes outside
+ * that format's range, with noise or with the power law).  Every other kind computes in FP32 registers: F32 stores f, the
  * shifted kinds store (f_i - omega_i rho0) * store_scale. */
 typedef enum {
     LBM_F64 = 0,

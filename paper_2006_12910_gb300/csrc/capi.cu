@@ -264,6 +264,26 @@ void fill_dom(DomDev& D, const lbm_params& p, int kind) {
     D.var = 3.0 * D.kT * (p.power_law ? 1.0 : D.inv_tau * (2.0 - D.inv_tau));
     D.var_f = (float)D.var; D.var_lo_f = (float)(D.var - (double)D.var_f);
     D.scale_f = (float)D.scale; D.inv_scale_f = (float)D.inv_scale;
+    {
+        // rho0 2^s in [2^60, 2^61)
+        int ex = 0;
+        std::frexp(p.rho0, &ex);
+        const int sh = 61 - ex;
+        const double tgx = p.tau * p.gx, tgy = p.tau * p.gy;
+        FixPrm& F = D.fix;
+        F.on = kind == LBM_F64 && sh > -900 && sh < 900 && p.tau > 0.50001 && std::fabs(tgx) < 0.49 && std::fabs(tgy) < 0.49;
+        if (F.on) {
+            auto split = [](int64_t x, int32_t& h, int32_t& l) {
+                l = (int32_t)(uint32_t)((uint64_t)x & 0xffffffffu);
+                h = (int32_t)((x - l) / ((int64_t)1 << 32));
+            };
+            F.e0 = 1086 - sh;
+            F.forced = tgx != 0.0 || tgy != 0.0;
+            split((int64_t)std::llround(std::ldexp(1.0 / p.tau, 62)), F.wh, F.wl);
+            split((int64_t)std::llround(std::ldexp(tgx, 64)), F.gxh, F.gxl);
+            split((int64_t)std::llround(std::ldexp(tgy, 64)), F.gyh, F.gyl);
+        }
+    }
     D.hot_d.omega = 1.0 / p.tau;
     D.hot_d.om = 1.0 - 1.0 / p.tau;
     D.hot_d.tgx = p.tau * p.gx;

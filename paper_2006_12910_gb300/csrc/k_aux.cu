@@ -1,8 +1,11 @@
 // k_aux.cu -- state set-up, conversion, moment output and global checks of
 // the GB300 D2Q9 library.  Off the per-step hot path except when a caller
 // asks for moments or checks.
+#include "collide_fix.cuh"
 #include "kernels.h"
 #include "lbm_dev.cuh"
+
+#include <cmath>
 
 namespace lbmk {
 
@@ -134,8 +137,10 @@ __global__ void k_moments(DomDev D, const typename S::T* arena, const uint8_t* s
 struct FF {
     float h, l;
 };
-struct MomPrm {  // rho0 and g / 2 as pairs, split on the host
+struct MomPrm {  // rho0 and g / 2 as pairs, split on the host; FP64 store: its fixed-point format (e0 0: none)
     FF rho0, gx2, gy2;
+    int32_t e0;
+    float unit;
 };
 __device__ __forceinline__ FF two_sum(float a, float b) {
     const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
@@ -148,6 +153,13 @@ __device__ __forceinline__ FF add(FF a, float b) {
 __device__ __forceinline__ FF add(FF a, FF b) {
     const FF s = two_sum(a.h, b.h);
     return FF{s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l))};
+}
+// A number of units of the fixed-point format as a pair.
+__device__ __forceinline__ FF pair_of(int64_t x) {
+    const float a = (float)(int32_t)(x >> 40) * 1099511627776.0f;  // 2^40
+    const float b = (float)((int32_t)(x >> 20) & 0xFFFFF) * 1048576.0f, c = (float)((int32_t)x & 0xFFFFF);
+    const FF s = two_sum(a, b);
+    return FF{s.h, __fadd_rn(s.l, c)};
 }
 // j / r - g2 (the velocity (j - r g / 2) / r) from the pairs, y about 1 / r:
 // the quotient's first digit and the remainder's, then the body-force term.
@@ -164,17 +176,20 @@ __device__ __forceinline__ float velocity(FF j, FF r, float y, FF g2) {
 // programmatic launch lets the launches over several domains follow one
 // another without the launch gap; each still waits for the one before it.
 // Bound by HBM (FP32 stores: 70 % of the copy rate) and, for the half-precision
-// and FP64 stores, by arithmetic.  Measured, launches back to back, against FP64
+// stores, by arithmetic.  Measured, launches back to back, against FP64
 // sums and divisions a node at a time: 2048x1024 shifted FP32 260 -> 20.9 us,
-// FP16 265 -> 17.3, FP64 191 -> 93; 96 ensemble domains (96 launches) 1812 -> 344;
+// FP16 265 -> 17.3, FP64 191 -> 33 (exact sums in the fixed-point
+// format of the collision); 96 ensemble domains (96 launches) 1812 -> 344;
 // 4096x2048 1023 -> 77.
+template <class S>
+__host__ __device__ constexpr int moment_chunk() { return sizeof(typename S::T) == 8 ? 2 : 4; }
 template <class S, bool ALIGNED>
 __global__ void __launch_bounds__(256) k_moments_f32(const __grid_constant__ DomDev D, const MomPrm P,
                                                      const typename S::T* arena, const uint8_t* solid, float* rho_o,
                                                      float* ux_o, float* uy_o) {
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    constexpr int V = S::V;
+    constexpr int V = moment_chunk<S>();
     typedef typename S::A A;
     const uint32_t chunks = (uint32_t)((D.nx + V - 1) / V), n = chunks * (uint32_t)D.ny;
     const uint32_t k = blockIdx.x * 256u + threadIdx.x;
@@ -184,7 +199,7 @@ __global__ void __launch_bounds__(256) k_moments_f32(const __grid_constant__ Dom
     const typename S::T* p = arena + D.off + ni;
     A f[9][V];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) load_vec<S>(p + (int64_t)i * D.plane, f[i], sizeof(A) == 4 ? (A)D.inv_scale_f : (A)1);
+    for (int i = 0; i < 9; ++i) load_vec<S, V>(p + (int64_t)i * D.plane, f[i], sizeof(A) == 4 ? (A)D.inv_scale_f : (A)1);
     uint8_t sol[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) sol[v] = solid[D.node_off + ni + v];
@@ -193,16 +208,19 @@ __global__ void __launch_bounds__(256) k_moments_f32(const __grid_constant__ Dom
     for (int v = 0; v < V; ++v) {
         bool plain;
         if constexpr (sizeof(A) == 8) {
-            // FP64 store: the sums stay in FP64 (two conversions, a Newton step for 1 / r and one FMA a component)
-            const double a = (f[1][v] + f[5][v]) + f[8][v], b = (f[3][v] + f[6][v]) + f[7][v];
-            const double c = (f[2][v] + f[5][v]) + f[6][v], d = (f[4][v] + f[7][v]) + f[8][v];
-            const double r = (f[0][v] + (f[2][v] + f[4][v])) + (a + b);
-            rho[v] = (float)r;
-            plain = rho[v] > 1e-30f && rho[v] < 1e30f;
-            const double y0 = (double)rcp_rho<float>(rho[v]);
-            const double yr = fma(y0, fma(-r, y0, 1.0), y0);
-            ux[v] = (float)fma(a - b, yr, -0.5 * D.gx);
-            uy[v] = (float)fma(c - d, yr, -0.5 * D.gy);
+            // FP64 store: exact sums in the fixed-point format of the collision
+            uint32_t t = 0;
+            int64_t g[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) g[i] = to_fix(f[i][v], P.e0, t);
+            const int64_t a = g[1] + g[5] + g[8], b = g[3] + g[6] + g[7];
+            const int64_t c = g[2] + g[5] + g[6], d = g[4] + g[7] + g[8];
+            const FF r = pair_of(g[0] + g[2] + g[4] + a + b);
+            const float rs = __fadd_rn(r.h, r.l), yr = rcp_rho<float>(rs);
+            rho[v] = rs * P.unit;
+            plain = P.e0 != 0 && t < FIX_RANGE && rho[v] > 1e-30f && rho[v] < 1e30f;
+            ux[v] = velocity(pair_of(a - b), r, yr, P.gx2);
+            uy[v] = velocity(pair_of(c - d), r, yr, P.gy2);
         } else {
             const FF a = add(two_sum(f[5][v], f[8][v]), f[1][v]), b = add(two_sum(f[6][v], f[7][v]), f[3][v]);
             const FF c = add(two_sum(f[5][v], f[6][v]), f[2][v]), d = add(two_sum(f[7][v], f[8][v]), f[4][v]);
@@ -338,10 +356,11 @@ template <class S>
 static cudaError_t launch_moments_f32(const DomDev& D, const void* arena, const uint8_t* solid, float* rho, float* ux,
                                       float* uy, cudaStream_t s) {
     // vector stores: every row of every output array starts on a chunk boundary
+    constexpr int V = moment_chunk<S>();
     const uintptr_t mis = (reinterpret_cast<uintptr_t>(rho) | reinterpret_cast<uintptr_t>(ux) |
-                           reinterpret_cast<uintptr_t>(uy)) % (S::V * sizeof(float));
-    const bool aligned = mis == 0 && D.nx % S::V == 0;
-    const int64_t n = (int64_t)((D.nx + S::V - 1) / S::V) * D.ny;
+                           reinterpret_cast<uintptr_t>(uy)) % (V * sizeof(float));
+    const bool aligned = mis == 0 && D.nx % V == 0;
+    const int64_t n = (int64_t)((D.nx + V - 1) / V) * D.ny;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((n + 255) / 256));
     cfg.blockDim = dim3(256);
@@ -356,7 +375,12 @@ static cudaError_t launch_moments_f32(const DomDev& D, const void* arena, const 
     cfg.attrs = at;
     cfg.numAttrs = st == cudaStreamCaptureStatusNone ? 1 : 0;
     auto pair = [](double v) { return FF{(float)v, (float)(v - (double)(float)v)}; };
-    const MomPrm P = {pair(D.rho0), pair(0.5 * D.gx), pair(0.5 * D.gy)};
+    MomPrm P = {pair(D.rho0), pair(0.5 * D.gx), pair(0.5 * D.gy), 0, 1.0f};
+    const int sh = 1086 - D.fix.e0;  // units of 2^-sh
+    if (D.fix.on && sh > 0 && sh < 120) {
+        P.e0 = D.fix.e0;
+        P.unit = std::ldexp(1.0f, -sh);
+    }
     const typename S::T* p = static_cast<const typename S::T*>(arena);
     return aligned ? cudaLaunchKernelEx(&cfg, k_moments_f32<S, true>, D, P, p, solid, rho, ux, uy)
                    : cudaLaunchKernelEx(&cfg, k_moments_f32<S, false>, D, P, p, solid, rho, ux, uy);

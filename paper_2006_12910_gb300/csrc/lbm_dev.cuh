@@ -86,16 +86,18 @@ template <> struct Vec<float2> {
 
 // ---------------------------------------------------------------------------
 // Population storage kinds.  V = consecutive nodes of one row a lane owns in
-// the register stream-collide kernel (one vector load or store of V*sizeof(T)
-// = 8 or 16 bytes per plane).  MINB / MINB_EXT: CTAs of 128 threads the
+// the register stream-collide kernel (one load or store of V*sizeof(T) = 8 or 16
+// bytes per plane).  MINB / MINB_EXT: CTAs of 128 threads the
 // register kernel asks to keep resident per SM (plain BGK / with noise or
 // the power law), which caps its registers per thread.
 // ---------------------------------------------------------------------------
+// FP64: one node a lane.  The pull needs no edge elements then, and the
+// fixed-point collision of a node leaves room for more warps.
 struct StF64 {
     typedef double T; typedef double A;
-    static constexpr int V = 2; static constexpr bool SHIFT = false; static constexpr bool SCALED = false;
+    static constexpr int V = 1; static constexpr bool SHIFT = false; static constexpr bool SCALED = false;
     static constexpr int KIND = 0;
-    static constexpr int MINB = 3, MINB_EXT = 3;
+    static constexpr int MINB = 8, MINB_EXT = 4;
 };
 struct StF32 {
     typedef float T; typedef float A;
@@ -134,17 +136,17 @@ __device__ __forceinline__ void from_a(float v, float, float& o) { o = v; }
 __device__ __forceinline__ void from_a(float v, float s, __half& o) { o = __float2half_rn(v * s); }
 __device__ __forceinline__ void from_a(float v, float s, __nv_bfloat16& o) { o = __float2bfloat16_rn(v * s); }
 
-// Vector load (read-only path) of V consecutive elements: one 8- or 16-byte access.
+// Vector load (read-only path) of NV consecutive elements: one 8- or 16-byte access.
 template <int B> struct VecOf;
 template <> struct VecOf<8> { typedef uint2 type; };
 template <> struct VecOf<16> { typedef uint4 type; };
-template <class S>
-__device__ __forceinline__ void load_vec(const typename S::T* p, typename S::A* out, typename S::A inv) {
-    typedef typename VecOf<S::V * sizeof(typename S::T)>::type VT;
-    union { VT u; typename S::T t[S::V]; } r;
+template <class S, int NV>
+__device__ __forceinline__ void load_vec(const typename S::T* p, typename S::A (&out)[NV], typename S::A inv) {
+    typedef typename VecOf<NV * sizeof(typename S::T)>::type VT;
+    union { VT u; typename S::T t[NV]; } r;
     r.u = __ldg(reinterpret_cast<const VT*>(p));
 #pragma unroll
-    for (int k = 0; k < S::V; ++k) out[k] = to_a(r.t[k], inv);
+    for (int k = 0; k < NV; ++k) out[k] = to_a(r.t[k], inv);
 }
 __device__ __forceinline__ uint32_t pack2(float a, float b, __half) {
     const __half2 h = __floats2half2_rn(a, b);
@@ -174,7 +176,7 @@ struct Chunk {  // as loaded; get() converts
 };
 template <class S>
 __device__ __forceinline__ void store_chunk(void* p, const typename ChunkOf<S>::W (&v)[ChunkOf<S>::N]) {
-    if constexpr (sizeof(typename S::T) == 8) *static_cast<double2*>(p) = make_double2(v[0], v[1]);
+    if constexpr (sizeof(typename S::T) == 8) *static_cast<double*>(p) = v[0];
     else if constexpr (sizeof(typename S::T) == 4) *static_cast<float4*>(p) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
     else *static_cast<uint2*>(p) = make_uint2(pack2(v[0].x, v[0].y, typename S::T()), pack2(v[1].x, v[1].y, typename S::T()));
 }
@@ -376,6 +378,12 @@ template <> __device__ __forceinline__ HotPrm<double> load_hot<double>(const Dom
     H.omega = a.x; H.om = a.y; H.tgx = b.x; H.tgy = b.y;
     H.rho0 = c.x; H.scale = c.y; H.inv_scale = d.x; H.pad = d.y;
     return H;
+}
+
+__device__ __forceinline__ FixPrm load_fix(const DomDev& D) {
+    const int4* p = reinterpret_cast<const int4*>(&D.fix);
+    const int4 a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + 2);
+    return FixPrm{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w};
 }
 
 template <typename A>

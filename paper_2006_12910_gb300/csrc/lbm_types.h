@@ -26,6 +26,16 @@ struct alignas(16) HotPrm {
     A omega, om, tgx, tgy, rho0, scale, inv_scale, pad;
 };
 
+// Fixed-point collision of the FP64 store (collide_fix.cuh): units of 2^-s,
+// e0 = 1086 - s; omega in units of 2^-62 and tau g in units of 2^-64, as halves
+// hi * 2^32 + lo with lo in [-2^31, 2^31).  on: the domain's parameters fit the
+// format; forced: tau g is not zero.
+struct alignas(16) FixPrm {
+    int32_t e0, on, forced, pad;
+    int32_t wh, wl, gxh, gxl;
+    int32_t gyh, gyl, pad2, pad3;
+};
+
 // One lattice domain as the kernels see it.  Populations of plane i live at
 // arena[off + i*plane + y*pitch + x]; with y walls each plane also holds one
 // ghost row on each side (y = -1 and y = ny, still addressed as off + i*plane
@@ -37,6 +47,7 @@ struct alignas(16) HotPrm {
 struct alignas(16) DomDev {
     HotPrm<double> hot_d;
     HotPrm<float> hot_f;
+    FixPrm fix;
     int32_t nx, ny, pitch, flags;
     int64_t off, plane, node_off, mask_off, item_off;
     int32_t seg_per_row, V;

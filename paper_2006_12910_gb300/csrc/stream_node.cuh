@@ -8,6 +8,7 @@
 #include <cstddef>
 
 #include "kernels.h"
+#include "collide_fix.cuh"
 #include "lbm_dev.cuh"
 
 namespace lbmk {
@@ -74,7 +75,9 @@ __device__ __forceinline__ void pull_rows(const Geo& G, int y, int& ym, int& yp)
 // V per-node flag words of one chunk (V*2 bytes, aligned).
 template <int V>
 __device__ __forceinline__ void load_flags(const uint16_t* p, uint16_t (&fl)[V]) {
-    if constexpr (V == 2) {
+    if constexpr (V == 1) {
+        fl[0] = __ldg(p);
+    } else if constexpr (V == 2) {
         const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(p));
         fl[0] = (uint16_t)w; fl[1] = (uint16_t)(w >> 16);
     } else if constexpr (V == 4) {
@@ -253,6 +256,29 @@ __device__ __forceinline__ bool finish_chunk(const StreamArgs& a, const DomDev& 
     typedef Vec<W> K;
     constexpr int V = S::V, N = K::N;
     uint32_t good = solid;
+    bool fix = false;
+    if constexpr (S::KIND == 0 && !NOISE && !PL) {
+        const FixPrm F = a.ndom == 1 ? a.dom0.fix : load_fix(D);
+        fix = F.on != 0;
+        if (fix) {
+#pragma unroll
+            for (int p = 0; p < V; ++p) {
+                double n9[9], out[9];
+#pragma unroll
+                for (int i = 0; i < 9; ++i) n9[i] = f[i][p];
+                bool ok = collide_fix(n9, out, F);
+                if (!ok && !((solid >> p) & 1u)) {
+                    ok = collide_f64(D, n9);
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) out[i] = n9[i];
+                }
+                if (ok) good |= 1u << p;
+#pragma unroll
+                for (int i = 0; i < 9; ++i) f[i][p] = out[i];
+            }
+        }
+    }
+    if (!fix)
 #pragma unroll
     for (int p = 0; p < ChunkOf<S>::N; ++p) {
         W n9[9];
