@@ -26,6 +26,8 @@
 //     items near the particle for step t+2;
 //  D. (launch 3) Eq. MP2 at t+2, which needs positions only.
 // At set-up the same roles run for the current step.
+#include <type_traits>
+
 #include "kernels.h"
 #include "lbm_dev.cuh"
 
@@ -390,7 +392,7 @@ union SmemU {
 // out, so each launch fetches only its own instructions); role0 >= LO picks
 // the first role of the launch.
 template <class S, int LO, int HI>
-__global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(PartArgs a, int modes, int role0) {
+__global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(const __grid_constant__ PartArgs a, int modes, int role0) {
     // A programmatic dependent launch waits here for the kernels before it
     // (completion and memory flush); otherwise this returns at once.
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -424,7 +426,10 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(P
     const int need = role == 0 ? (PL_FORCES | PL_SWAP) : role == 1 ? PL_LJ : role == 2 ? PL_RASTER : PL_MARK;
     if (!(modes & need)) return;
     if (st.dom < 0) return;
-    const DomDev D = a.one_domain ? a.dom0 : a.doms[st.dom];  // one domain: from the launch parameters
+    // One domain: the descriptor in the launch parameters.  Role A keeps the fields
+    // it uses in registers; the other roles pass the descriptor to functions, and
+    // a copy would put all of it (0.6 KB) into every thread's local memory.
+    typename std::conditional<HI == 0, const DomDev, const DomDev&>::type D = a.one_domain ? a.dom0 : a.doms[st.dom];
     if (p - D.p0 >= D.np) return;
     const int par = (int)(t & 1);
     const PartState* S0 = a.state + (int64_t)par * a.np;
