@@ -225,6 +225,10 @@ void fill_dom(DomDev& D, const lbm_params& p, int kind) {
         const uint64_t d = (uint64_t)D.seg_per_row, items = (uint64_t)p.ny * d;
         D.spr_magic = (d > 1 && items * d < ((uint64_t)1 << 32)) ? (uint32_t)(((uint64_t)1 << 32) / d + 1) : 0u;
     }
+    {
+        const uint64_t d = (uint64_t)D.pitch / 16, n = (uint64_t)D.pitch * p.ny / 16;
+        D.pitch_magic = (d > 1 && n * d < ((uint64_t)1 << 32)) ? (uint32_t)(((uint64_t)1 << 32) / d + 1) : 0u;
+    }
     D.seed = p.seed;
     D.domain_id = p.domain_id;
     D.tau = p.tau;

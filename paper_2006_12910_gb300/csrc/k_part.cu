@@ -440,7 +440,6 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(c
 
     __shared__ __align__(16) unsigned char smem_raw[sizeof(SmemU)];
     SmemU& sm = *reinterpret_cast<SmemU*>(smem_raw);
-    __shared__ double tot[DIAG_N];
     __shared__ int lj_n, nnear;
     __shared__ int sh_warp[MAX_WARPS];
     __shared__ long long sh_warp2[MAX_WARPS];
@@ -474,31 +473,119 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(c
         // - 2 fy S_x with S = sum f' e_k: three FP64 additions per link.
         // Each warp sums its own terms by shuffles in a fixed order and the
         // warps are added in a fixed order, so the totals are deterministic.
+        // A warp's FP64 instruction occupies its scheduler's FP64 unit for about
+        // 70 cycles whatever the number of active lanes, so phase 2 runs on the
+        // lanes of warp 0 with one chain of operations for the nine entries of
+        // M + Z/2 and of the right-hand side, and lanes 0-2 solve a row each (20
+        // instructions on the path, one thread had about 100); what needs no
+        // link sum is computed before them.  With the link nodes' division by
+        // the pitch as a multiply-high and the decoded links kept from phase 1 to
+        // phase 3 the launch takes 12.3 us in sequence (14.3 before).
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
         __shared__ double wsa[A_BLOCK / 32][DIAG_N];  // per-warp partial sums
         __shared__ int wsi[4][5];                     // per-warp integer sums Ixx, Ixy, Iyy, J1, J2
         __shared__ long long wsk[4];                  // per-warp integer sum K
-        __shared__ double xmid[3];
+        __shared__ double vals[20];                   // totals 0-12, integer sums 13-18 as doubles, 0
+        __shared__ double sys[9];                     // M + Z/2 (upper triangle) and the right-hand side
+        __shared__ double newst[6], xmid[3], zval[6];
         const int32_t* links = a.links + (int64_t)par * a.links_total;
         const int32_t* flips = a.flips + (int64_t)par * a.flips_total;
         const int nl = nl2[par], nf = nf2[par];
+        const bool forces = modes & PL_FORCES, swap = modes & PL_SWAP;
+        // one round of four links per thread covers nl <= 512: the decoded links
+        // and slot values then stay in registers from phase 1 to phase 3
+        const bool one_round = nl <= 4 * 128;
+        int32_t ent[4] = {0, 0, 0, 0};
+        if (warp < 4) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int l = (int)threadIdx.x + 128 * u;
+                if (l < nl) ent[u] = links[st.link_off + l];
+            }
+        }
         // the Eq. MP2 sums of t, loaded now by the threads that add them up
         double ljc = 0.0;
         if (threadIdx.x >= 6 && threadIdx.x < 9 && D.lj_psi != 0.0 && D.lj_rit > 0.0)
             ljc = a.ljf[4 * ((int64_t)par * a.np + p) + (threadIdx.x - 6)];
-        const bool forces = modes & PL_FORCES, swap = modes & PL_SWAP;
         double acc[DIAG_N];
 #pragma unroll
         for (int c = 0; c < DIAG_N; ++c) acc[c] = 0.0;
-        const A scl = (A)D.scale, inv = (A)D.inv_scale;
+        const A scl = (A)(sizeof(A) == 4 ? D.scale_f : D.scale), inv = (A)(sizeof(A) == 4 ? D.inv_scale_f : D.inv_scale);
         // integer node of the centre and the fractional offset
         const double fl_x = floor(q.x), fl_y = floor(q.y);
         const int ix = (int)fl_x, iy = (int)fl_y;
         const double fxd = q.x - fl_x, fyd = q.y - fl_y;
-        // one round of four links per thread covers nl <= 512: the slot
-        // values then stay in registers from phase 1 to phase 3
-        const bool one_round = nl <= 4 * 128;
+        // A link: its direction k, 2 x (arm x e_k) from the integer parts, and the
+        // offsets of the slots that r_v + e_k (ia) and r_v (ib) pull next.
+        auto decode = [&](int32_t e, int& k, int& a2, int64_t& ia, int64_t& ib) {
+            const int node = e >> 3;
+            k = (e & 7) + 1;
+            const int vy = D.pitch_magic ? (int)__umulhi((uint32_t)node >> 4, D.pitch_magic) : node / D.pitch;
+            const int vx = node - vy * D.pitch;
+            int fx = vx + cx(k), fy = vy + cy(k);
+            wrap_node(D, fx, fy);
+            const int mx2 = 2 * wrap_off(vx - ix, D.nx, px) + cx(k);
+            const int my2 = 2 * wrap_off(vy - iy, D.ny, py) + cy(k);
+            a2 = mx2 * cy(k) - my2 * cx(k);
+            ia = (int64_t)k * D.plane + node;
+            ib = (int64_t)opp(k) * D.plane + (int64_t)fy * D.pitch + fx;
+        };
         A va[4], vb[4];
+        int kk[4], a2s[4];
+        int64_t ias[4], ibs[4];
+        // Warp 0, for phase 2: the lane's coefficients and the part of its entry
+        // that needs no sum.  Lanes 0-5: the entries xx, xy, xO, yy, yO, OO of
+        // M + Z/2, Z = rho0/6 x (integer sums with the fractional offset applied);
+        // lanes 6-8: M X(t) + G/2, G = motion-independent force and torque +
+        // buoyancy term; lanes 9-14: the position, the angle and the old velocities.
+        double cf[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0}, cw = 0.0, cb = 0.0;
+        int vi[6] = {19, 19, 19, 19, 19, 19};
+        if (warp == 0) {
+            const double r12 = D.rho0 * (1.0 / 12.0);
+            if (lane < 6) {
+                cw = r12;
+                cb = (lane == 0 || lane == 3) ? st.m : (lane == 5 ? st.I : 0.0);
+                cf[0] = lane == 5 ? 0.25 : ((lane & 1) == 0 && lane ? 0.5 : 1.0);
+                vi[0] = lane == 2 ? 16 : (lane == 3 ? 15 : 13 + lane);  // Ixx Ixy J1 Iyy J2 K
+                if (lane == 2 || lane == 4 || lane == 5) {
+                    cf[1] = -fxd;
+                    cf[2] = fyd;
+                    vi[1] = lane == 2 ? 14 : (lane == 4 ? 15 : 17);  // Ixy Iyy J2
+                    vi[2] = lane == 2 ? 13 : (lane == 4 ? 14 : 16);  // Ixx Ixy J1
+                }
+                if (lane == 5) {
+                    cf[3] = fxd * fxd;
+                    cf[4] = -2.0 * fxd * fyd;
+                    cf[5] = fyd * fyd;
+                    vi[3] = 15;
+                    vi[4] = 14;
+                    vi[5] = 13;
+                }
+            } else if (lane < 9) {
+                const int c = lane - 6;
+                cw = 1.0;
+                const double v = c == 0 ? q.U : (c == 1 ? q.V : q.Om), g = c == 0 ? D.gx : (c == 1 ? D.gy : 0.0);
+                cb = (c == 2 ? st.I : st.m) * v + 0.5 * (st.m * st.buoy * g);
+                cf[0] = c == 2 ? -0.5 : -1.0;  // half of -2 S, and of -sum f' A + 2 fx S_y - 2 fy S_x
+                vi[0] = c;
+                if (c == 2) {
+                    cf[1] = fxd;
+                    cf[2] = -fyd;
+                    vi[1] = 1;
+                    vi[2] = 0;
+                }
+                cf[3] = cf[4] = 0.5;
+                vi[3] = 3 + c;
+                vi[4] = 6 + c;
+            } else if (lane == 9 && advance) {
+                // r_c(t+1) = r_c(t) + U_p(t) and the angle likewise
+                double x1, y1;
+                next_position(D, q, st.fixed, x1, y1);
+                newst[0] = x1;
+                newst[1] = y1;
+                newst[5] = st.fixed ? q.th : q.th + q.Om;
+            }
+        }
         if (warp < 4) {
             int Ixx = 0, Ixy = 0, Iyy = 0, J1 = 0, J2 = 0;
             long long K = 0;
@@ -507,22 +594,14 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(c
                 // flight before any is used
 #pragma unroll 1
                 for (int l0 = threadIdx.x; l0 < nl; l0 += 4 * 128) {
-                    int kk[4], a2s[4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         const int l = l0 + 128 * u;
-                        const int32_t e = l < nl ? links[st.link_off + l] : 0;
-                        const int node = e >> 3, k = (e & 7) + 1;
-                        const int vy = node / D.pitch, vx = node - vy * D.pitch;
-                        int fx = vx + cx(k), fy = vy + cy(k);
-                        wrap_node(D, fx, fy);
-                        kk[u] = k;
-                        const int mx2 = 2 * wrap_off(vx - ix, D.nx, px) + cx(k);
-                        const int my2 = 2 * wrap_off(vy - iy, D.ny, py) + cy(k);
-                        a2s[u] = mx2 * cy(k) - my2 * cx(k);
+                        if (!one_round) ent[u] = l < nl ? links[st.link_off + l] : 0;
                         if (l < nl) {
-                            va[u] = to_a(base[(int64_t)k * D.plane + node], inv);
-                            vb[u] = to_a(base[(int64_t)opp(k) * D.plane + (int64_t)fy * D.pitch + fx], inv);
+                            decode(ent[u], kk[u], a2s[u], ias[u], ibs[u]);
+                            va[u] = to_a(base[ias[u]], inv);
+                            vb[u] = to_a(base[ibs[u]], inv);
                         }
                     }
 #pragma unroll
@@ -602,106 +681,106 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(c
             }
         }
         __syncthreads();
-        __shared__ long long itot[6];
-        if (forces && threadIdx.x < DIAG_N) {
-            // component groups: link sums 0-2 (warps 0-3), covered/uncovered 3-5
-            // and 9-12 (warp 4), LJ 6-8 (role D, earlier launch); fixed order
-            const int c = threadIdx.x;
-            double x = 0.0;
-            if (c < 3) x = ((wsa[0][c] + wsa[1][c]) + wsa[2][c]) + wsa[3][c];
-            else if (c < 6 || c >= 9) x = wsa[4][c];
-            else x = ljc;
-            tot[c] = x;
-            if (c >= 3) a.diag[(int64_t)p * DIAG_N + c] = x;
-        } else if (forces && threadIdx.x >= 32 && threadIdx.x < 38) {
-            const int c = threadIdx.x - 32;
-            itot[c] = c < 5 ? (long long)wsi[0][c] + wsi[1][c] + wsi[2][c] + wsi[3][c]
-                            : wsk[0] + wsk[1] + wsk[2] + wsk[3];
-        }
-        __syncthreads();
-        __shared__ double zsh[6], f0sh[3];
-        if (threadIdx.x == 0) {
-            // Eqs. MP5, MP6 (velocities) with r_c(t+1) = r_c(t) + U_p(t).  One
-            // thread, FP64: the dependent chain is kept short (one reciprocal).
-            PartState n = q;
-            double xm[3] = {q.U, q.V, q.Om};
-            double F0x = 0.0, F0y = 0.0, T0 = 0.0, z[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-            if (forces) {
-                // the motion-independent link force and torque
-                F0x = -2.0 * tot[0];
-                F0y = -2.0 * tot[1];
-                T0 = -tot[2] + 2.0 * fxd * tot[1] - 2.0 * fyd * tot[0];
-                // Z = rho0/6 x (integer sums with the fractional offset applied)
-                const double Ixx = (double)itot[0], Ixy = (double)itot[1], Iyy = (double)itot[2];
-                const double J1 = (double)itot[3], J2 = (double)itot[4], Kd = (double)itot[5];
-                const double r6 = D.rho0 / 6.0;
-                z[0] = r6 * Ixx;
-                z[1] = r6 * Ixy;
-                z[2] = r6 * (0.5 * J1 - fxd * Ixy + fyd * Ixx);
-                z[3] = r6 * Iyy;
-                z[4] = r6 * (0.5 * J2 - fxd * Iyy + fyd * Ixy);
-                z[5] = r6 * (0.25 * Kd - (fxd * J2 - fyd * J1) + fxd * fxd * Iyy - 2.0 * fxd * fyd * Ixy +
-                             fyd * fyd * Ixx);
+        if (warp == 0) {
+            if (forces && lane < DIAG_N) {
+                // component groups: link sums 0-2 (warps 0-3), covered/uncovered 3-5
+                // and 9-12 (warp 4), LJ 6-8 (role D, earlier launch); fixed order
+                const int c = lane;
+                double x = 0.0;
+                if (c < 3) x = ((wsa[0][c] + wsa[1][c]) + wsa[2][c]) + wsa[3][c];
+                else if (c < 6 || c >= 9) x = wsa[4][c];
+                else x = ljc;
+                vals[c] = x;
+                if (c >= 3) a.diag[(int64_t)p * DIAG_N + c] = x;
+            } else if (forces && lane < 19) {
+                const int c = lane - 13;
+                vals[lane] = (double)(c < 5 ? (long long)wsi[0][c] + wsi[1][c] + wsi[2][c] + wsi[3][c]
+                                            : wsk[0] + wsk[1] + wsk[2] + wsk[3]);
+            } else if (lane < 20) {
+                vals[lane] = 0.0;
+                if (!forces && lane >= 13) vals[lane - 13] = 0.0;
             }
-            if (advance && !st.fixed) {
-                if (forces) {
-                    // G = motion-independent force and torque + buoyancy term
-                    const double G0 = (F0x + tot[3]) + tot[6] + st.m * st.buoy * D.gx;
-                    const double G1 = (F0y + tot[4]) + tot[7] + st.m * st.buoy * D.gy;
-                    const double G2 = (T0 + tot[5]) + tot[8];
+            if (!forces && lane < 13) vals[lane] = 0.0;
+            __syncwarp();
+            if (lane < 9) {
+                double v = cf[0] * vals[vi[0]];
+#pragma unroll
+                for (int m = 1; m < 6; ++m) v = fma(cf[m], vals[vi[m]], v);
+                sys[lane] = fma(cw, v, cb);
+                if (lane < 6) zval[lane] = 2.0 * (cw * v);
+            }
+            __syncwarp();
+            const bool move = advance && !st.fixed, solve = move && forces;
+            bool fine = true;
+            double xm = 0.0, vn = 0.0;
+            if (lane < 3) {
+                xm = vn = lane == 0 ? q.U : (lane == 1 ? q.V : q.Om);
+                if (solve) {
                     // (M + Z/2) X_mid = M X(t) + G/2, M + Z/2 symmetric positive
-                    // definite: X_mid = adj(M + Z/2) r / det(M + Z/2)
-                    const double a00 = st.m + 0.5 * z[0], a01 = 0.5 * z[1], a02 = 0.5 * z[2];
-                    const double a11 = st.m + 0.5 * z[3], a12 = 0.5 * z[4], a22 = st.I + 0.5 * z[5];
-                    const double c00 = a11 * a22 - a12 * a12, c01 = a02 * a12 - a01 * a22, c02 = a01 * a12 - a02 * a11;
-                    const double c11 = a00 * a22 - a02 * a02, c12 = a01 * a02 - a00 * a12, c22 = a00 * a11 - a01 * a01;
-                    const double inv_det = 1.0 / (a00 * c00 + a01 * c01 + a02 * c02);
-                    const double r0 = st.m * q.U + 0.5 * G0, r1 = st.m * q.V + 0.5 * G1, r2 = st.I * q.Om + 0.5 * G2;
-                    xm[0] = (c00 * r0 + c01 * r1 + c02 * r2) * inv_det;
-                    xm[1] = (c01 * r0 + c11 * r1 + c12 * r2) * inv_det;
-                    xm[2] = (c02 * r0 + c12 * r1 + c22 * r2) * inv_det;
-                    n.U = 2.0 * xm[0] - q.U;
-                    n.V = 2.0 * xm[1] - q.V;
-                    n.Om = 2.0 * xm[2] - q.Om;
+                    // definite: row `lane` of adj(M + Z/2) r / det(M + Z/2), the
+                    // determinant expanded along that row
+                    const int i = lane, j = i == 2 ? 0 : i + 1, l = i == 0 ? 2 : i - 1;  // cyclic
+                    auto at = [&](int r, int c) { return sys[r <= c ? (r == 0 ? c : r + c + 1) : (c == 0 ? r : r + c + 1)]; };
+                    const double aii = at(i, i), aij = at(i, j), ail = at(i, l), ajj = at(j, j), ajl = at(j, l), all = at(l, l);
+                    const double cii = fma(ajj, all, -(ajl * ajl)), cij = fma(ajl, ail, -(aij * all)),
+                                 cil = fma(aij, ajl, -(ail * ajj));
+                    const double det = fma(ail, cil, fma(aij, cij, aii * cii));
+                    const double num = fma(cil, sys[6 + l], fma(cij, sys[6 + j], cii * sys[6 + i]));
+                    // 1 / det: the hardware approximation times 1 + e + e^2, and the
+                    // quotient corrected by its remainder (the division far from 1)
+                    double y;
+                    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(det));
+                    const int ex = (__double2hiint(det) >> 20) & 0x7ff;
+                    if (ex > 200 && ex < 1800) {
+                        const double e = fma(-det, y, 1.0);
+                        y = fma(y, fma(e, e, e), y);
+                        const double x0 = num * y;
+                        xm = fma(fma(-det, x0, num), y, x0);
+                    } else {
+                        xm = num * (1.0 / det);
+                    }
+                    vn = fma(2.0, xm, -vn);
                 }
-                next_position(D, q, false, n.x, n.y);
-                n.th = q.th + q.Om;
                 // A particle faster than a node per step, or a state that is no
                 // longer finite (an unstable lattice around it), is an error; the
                 // particle then stays where it was, at rest, so that later
                 // launches keep rasterising a finite disk inside the domain.
-                const bool ok = fabs(n.U) < 1.0 && fabs(n.V) < 1.0 && fabs(n.Om) < 1.0 && isfinite(n.x) &&
-                                isfinite(n.y) && isfinite(n.th);
-                if (!ok) {
+                const double pos = newst[lane == 2 ? 5 : lane];
+                const uint32_t hv = (uint32_t)__double2hiint(vn) & 0x7fffffffu, hp = (uint32_t)__double2hiint(pos) & 0x7fffffffu;
+                fine = !move || (hv < 0x3ff00000u && hp < 0x7ff00000u);  // |v| < 1, finite
+            }
+            if (!__all_sync(0xffffffffu, fine)) {
+                if (lane == 0) {
                     atomicOr(a.err, ERR_STATE);
-                    n = q;
-                    n.U = n.V = n.Om = 0.0;
-                    xm[0] = xm[1] = xm[2] = 0.0;
+                    newst[0] = q.x;
+                    newst[1] = q.y;
+                    newst[5] = q.th;
                 }
+                xm = vn = 0.0;
             }
-            if (advance) {
-                a.state[(int64_t)(par ^ 1) * a.np + p] = n;
-                if (a.rec) a.rec[((t + 1) % a.rec_cap) * a.np + p] = n;
+            if (lane < 3) {
+                xmid[lane] = xm;
+                newst[2 + lane] = vn;
             }
-#pragma unroll
-            for (int c = 0; c < 6; ++c) zsh[c] = z[c];
-            f0sh[0] = F0x;
-            f0sh[1] = F0y;
-            f0sh[2] = T0;
-            xmid[0] = xm[0];
-            xmid[1] = xm[1];
-            xmid[2] = xm[2];
+            __syncwarp();
+            if (advance && lane < 6)
+                reinterpret_cast<double*>(a.state + (int64_t)(par ^ 1) * a.np + p)[lane] = newst[lane];
         }
         __syncthreads();
         // the stream-collide pass after this launch may be placed on the SMs
         // now; it waits for this launch's completion before it reads
         asm volatile("griddepcontrol.launch_dependents;");
-        if (forces && warp == 4 && lane < 3) {
-            // the link force of Eq. MP1 at the mid-step boundary velocity, beside the exchange
-            const int c = lane;
-            const int i0 = c == 0 ? 0 : (c == 1 ? 1 : 2), i1 = c == 0 ? 1 : (c == 1 ? 3 : 4),
-                      i2 = c == 0 ? 2 : (c == 1 ? 4 : 5);
-            a.diag[(int64_t)p * DIAG_N + c] = f0sh[c] - (zsh[i0] * xmid[0] + zsh[i1] * xmid[1] + zsh[i2] * xmid[2]);
+        if (warp == 4) {
+            if (forces && lane < 3) {
+                // the link force of Eq. MP1 at the mid-step boundary velocity, beside the exchange
+                const int c = lane;
+                const int i0 = c == 0 ? 0 : (c == 1 ? 1 : 2), i1 = c == 0 ? 1 : (c == 1 ? 3 : 4),
+                          i2 = c == 0 ? 2 : (c == 1 ? 4 : 5);
+                const double f0 = c == 2 ? -vals[2] + 2.0 * fxd * vals[1] - 2.0 * fyd * vals[0] : -2.0 * vals[c];
+                a.diag[(int64_t)p * DIAG_N + c] = f0 - (zval[i0] * xmid[0] + zval[i1] * xmid[1] + zval[i2] * xmid[2]);
+            }
+            if (advance && a.rec && lane < 6)
+                reinterpret_cast<double*>(a.rec + ((t + 1) % a.rec_cap) * a.np + p)[lane] = newst[lane];
         }
         if (swap && warp < 4) {
             // Eqs. MP7-MP8 as a pre-stream exchange with u_b at mid-step:
@@ -715,28 +794,17 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(c
                 for (int u = 0; u < 4; ++u) {
                     const int l = l0 + 128 * u;
                     if (l >= nl) break;
-                    const int32_t e = links[st.link_off + l];
-                    const int node = e >> 3, k = (e & 7) + 1;
-                    const int vy = node / D.pitch, vx = node - vy * D.pitch;
-                    int fx = vx + cx(k), fy = vy + cy(k);
-                    wrap_node(D, fx, fy);
-                    typename S::T* sa = base + (int64_t)k * D.plane + node;                          // pulled by r_v + e_k
-                    typename S::T* sb = base + (int64_t)opp(k) * D.plane + (int64_t)fy * D.pitch + fx;  // pulled by r_v
-                    A xa, xb;
-                    if (one_round && forces) {
-                        xa = va[u];
-                        xb = vb[u];
-                    } else {
-                        xa = to_a(*sa, inv);
-                        xb = to_a(*sb, inv);
+                    if (!(one_round && forces)) {
+                        decode(links[st.link_off + l], kk[u], a2s[u], ias[u], ibs[u]);
+                        va[u] = to_a(base[ias[u]], inv);
+                        vb[u] = to_a(base[ibs[u]], inv);
                     }
-                    const int mx2 = 2 * wrap_off(vx - ix, D.nx, px) + cx(k);
-                    const int my2 = 2 * wrap_off(vy - iy, D.ny, py) + cy(k);
-                    const A arm = (A)0.5 * (A)(mx2 * cy(k) - my2 * cx(k)) - (fxa * (A)cy(k) - fya * (A)cx(k));
+                    const int k = kk[u];
+                    const A arm = (A)0.5 * (A)a2s[u] - (fxa * (A)cy(k) - fya * (A)cx(k));
                     const A ube = Um * (A)cx(k) + Vm * (A)cy(k) + Om * arm;
                     const A corr = r6a * (A)wgt(k) * ube;
-                    from_a(xb + corr, scl, *sa);
-                    from_a(xa - corr, scl, *sb);
+                    from_a(vb[u] + corr, scl, base[ias[u]]);
+                    from_a(va[u] - corr, scl, base[ibs[u]]);
                 }
             }
         }

@@ -57,7 +57,10 @@ struct alignas(16) DomDev {
     // every item of the domain), else local / seg_per_row
     uint32_t spr_magic;
     uint64_t seed;
-    uint32_t domain_id, pad1;
+    uint32_t domain_id;
+    // node -> row: y = umulhi(node >> 4, pitch_magic) when nonzero (exact for every
+    // node of the domain; pitch is a multiple of 16), else node / pitch
+    uint32_t pitch_magic;
     double tau, inv_tau, rho0, gx, gy;
     double rho_in, rho_out, drho_in, drho_out;  // open-column densities (and minus rho0)
     double kT;
