@@ -130,7 +130,7 @@ static __device__ __noinline__ bool collide_f64(const DomDev& D, double* f) {
 #pragma unroll
     for (int i = 0; i < 9; ++i) n9[i] = f[i];
     const HotPrm<double> H = load_hot<double>(D);
-    const double rho = collide_nodes<double, false, false, false>(n9, H, ExtPrm<double>{}, none);
+    const double rho = collide_nodes<double, false, false, false>(n9, H, ExtPrm<double>{}, none, 0.0);
 #pragma unroll
     for (int i = 0; i < 9; ++i) f[i] = n9[i];
     return rho_ok(rho);

@@ -237,9 +237,6 @@ __device__ __forceinline__ W sqrt_hw(W x) {
     const W r = vmul(x, y);
     return vfma(vfma(vmul(K::all(-1.0f), r), r, x), vmul(K::all(0.5f), y), r);
 }
-__device__ __forceinline__ float vabs(float x) { return fabsf(x); }
-__device__ __forceinline__ float2 vabs(float2 x) { return make_float2(fabsf(x.x), fabsf(x.y)); }
-
 // 2 ln u of the uniform with mantissa bits m in [1, 2) as above: u = 2^e (1 + f)
 // with 1 + f in [sqrt(1/2), sqrt 2), ln(1 + f) = f + f^2 (f p(f) - 1/2), p the
 // degree-7 minimax polynomial of (ln(1 + f) - f + f^2 / 2) / f^3 on that interval
@@ -457,7 +454,7 @@ template <> __device__ __forceinline__ float divn<float>(float a, float b) { ret
 template <> __device__ __forceinline__ double divn<double>(double a, double b) { return a / b; }
 
 template <typename A>
-__device__ __noinline__ A solve_tau_pl(A Astr, ExtPrm<A> P) {
+__device__ __forceinline__ A solve_tau_pl(A Astr, const ExtPrm<A>& P) {
     const A n = P.n, tmin = P.tmin, tmax = P.tmax;
     if (P.n_is_one) {
         A t = (A)0.5 + (A)3.0 * P.xi;
@@ -484,86 +481,52 @@ __device__ __noinline__ A solve_tau_pl(A Astr, ExtPrm<A> P) {
     return t;
 }
 
-// tau* of the nodes of W.  FP32: Newton from 1/2 + c (t^(1-n) = 1) instead of the
-// far bracket end, the nodes of a pair in step and without branches per node.
-// The first step is taken in the form t (1/2 + n q) / (t - (1-n) q), q = c t^(1-n);
-// the others subtract g / g', whose rounding vanishes with g, until a step is
-// below 2.5e-4 t, when what is left is a few parts in 1e8 (g'' t / (2 g') is below
-// 1 over n in [0.1, 3], 0.1 at n = 0.75).  Two or three evaluations of t^(1-n)
-// where the monotone iteration took five to eight; a node that does not get there
-// in six (a start beyond the turning point of g, far clamps) takes that one.
-// Power law n = 0.75, 2048x1024 shifted FP32: 36.4 -> 27.0 us a step; n = 1.5
-// (clamped nearly everywhere) 26.8 -> 24.8.
-__device__ __forceinline__ float lg2_hw(float x) {
-    float y;
-    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ float ex2_hw(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-template <class W>
-__device__ __forceinline__ W solve_taus(W astr, const ExtPrm<typename Vec<W>::A>& P) {
-    typedef Vec<W> K;
-    W tau;
-    if constexpr (sizeof(typename K::A) == 8) {
-        tau = solve_tau_pl<double>(astr, P);
-    } else {
-        const float n = P.n, om = 1.0f - n, tmin = P.tmin, tmax = P.tmax;
-        W t, c, q, den;
-        bool set[K::N];  // no iteration: n = 1, no strain or a clamp
-        bool open = false;
+// tau* of NN nodes.  FP32: the iteration of solve_tau_pl on all of them in step,
+// so that their logarithms, exponentials and divisions overlap and a warp runs
+// as many iterations as its slowest node needs once, not node after node
+// (power law n = 0.75, 2048x1024 shifted FP32: 36.4 -> 30.8 us a step).  Every
+// node takes exactly the values solve_tau_pl gives it: where the strain is
+// small a last-place difference of tau* grows by 10^3 within 100 steps.  (Newton
+// from a near start, three evaluations a node, took 27.0 us and lost that.)
+template <int NN>
+__device__ __forceinline__ void solve_taus(const double (&astr)[NN], const ExtPrm<double>& P, double (&tau)[NN]) {
 #pragma unroll
-        for (int k = 0; k < K::N; ++k) {
-            const float a = K::get(astr, k), ck = 3.0f * P.xi * ex2_hw((n - 1.0f) * lg2_hw(a));
-            const bool low = P.n_is_one ? false : (a > 0.0f ? tmin - 0.5f - ck * P.tmin_pow >= 0.0f : n >= 1.0f);
-            const bool high = P.n_is_one ? false : (a > 0.0f ? tmax - 0.5f - ck * P.tmax_pow <= 0.0f : n < 1.0f);
-            set[k] = P.n_is_one || low || high;
-            const float t0 = low ? tmin : (high ? tmax : fminf(fmaxf(0.5f + (P.n_is_one ? 3.0f * P.xi : ck), tmin), tmax));
-            K::set(t, k, t0);
-            K::set(c, k, set[k] ? 0.0f : ck);
-            open |= !set[k];
-        }
-        tau = t;
-        if (open) {
+    for (int k = 0; k < NN; ++k) tau[k] = solve_tau_pl<double>(astr[k], P);
+}
+template <int NN>
+__device__ __forceinline__ void solve_taus(const float (&astr)[NN], const ExtPrm<float>& P, float (&tau)[NN]) {
+    const float n = P.n, tmin = P.tmin, tmax = P.tmax, om = 1.0f - n;
+    float c[NN];
+    bool open[NN], any = false;
+#pragma unroll
+    for (int k = 0; k < NN; ++k) {
+        c[k] = __fmul_rn(3.0f * P.xi, powa<float>(astr[k], n - 1.0f));
+        const bool low = astr[k] > 0.0f ? tmin - 0.5f - c[k] * P.tmin_pow >= 0.0f : n >= 1.0f;
+        const bool high = astr[k] > 0.0f ? tmax - 0.5f - c[k] * P.tmax_pow <= 0.0f : n < 1.0f;
+        if (P.n_is_one) tau[k] = fminf(fmaxf(0.5f + 3.0f * P.xi, tmin), tmax);
+        else tau[k] = low ? tmin : (high ? tmax : (n < 1.0f ? tmax : tmin));
+        open[k] = !P.n_is_one && !low && !high;
+        any |= open[k];
+    }
 #pragma unroll 1
-            for (int it = 0;; ++it) {
+    for (int it = 0; any && it < 60; ++it) {
+        any = false;
+        float p[NN];
 #pragma unroll
-                for (int k = 0; k < K::N; ++k) K::set(q, k, ex2_hw(om * lg2_hw(K::get(t, k))));
-                q = vmul(c, q);
-                den = vfma(q, K::all(-om), t);
-                W r;
+        for (int k = 0; k < NN; ++k) p[k] = powa<float>(tau[k], om);
 #pragma unroll
-                for (int k = 0; k < K::N; ++k) K::set(r, k, rcp_rho<float>(K::get(den, k)));
-                r = vmul(t, r);  // 1 / g'
-                bool more = false;
-                if (it == 0) {
-                    t = vmul(vfma(K::all(n), q, K::all(0.5f)), r);
-                    more = true;
-                } else {
-                    const W d = vmul(vsub(vadd(t, K::all(-0.5f)), q), r);
-                    t = vsub(t, d);
-#pragma unroll
-                    for (int k = 0; k < K::N; ++k)
-                        more |= !set[k] && !(fabsf(K::get(d, k)) <= 2.5e-4f * K::get(t, k) && K::get(den, k) > 0.0f);
-                }
-#pragma unroll
-                for (int k = 0; k < K::N; ++k) K::set(t, k, fminf(fmaxf(K::get(t, k), tmin), tmax));
-                if (!more) break;
-                if (it == 6) {
-#pragma unroll
-                    for (int k = 0; k < K::N; ++k) K::set(t, k, solve_tau_pl<float>(K::get(astr, k), P));
-                    break;
-                }
+        for (int k = 0; k < NN; ++k) {
+            const float t = tau[k];
+            const float g = __fmaf_rn(-c[k], p[k], t - 0.5f);
+            const float dg = 1.0f - __fdividef(__fmul_rn(__fmul_rn(c[k], om), p[k]), t);
+            const float tn = fminf(fmaxf(t - __fdividef(g, dg), tmin), tmax);
+            if (open[k]) {
+                tau[k] = tn;
+                open[k] = !(fabsf(tn - t) <= 2e-7f * t);
+                any |= open[k];
             }
-#pragma unroll
-            for (int k = 0; k < K::N; ++k)
-                if (!set[k]) K::set(tau, k, K::get(t, k));
         }
     }
-    return tau;
 }
 
 // ---------------------------------------------------------------------------
@@ -581,8 +544,9 @@ __device__ __forceinline__ W solve_taus(W astr, const ExtPrm<typename Vec<W>::A>
 // whose rounding error stays at the scale of f_i rather than of omega f_i.
 // Returns false when rho is not a positive finite number.
 // ---------------------------------------------------------------------------
-// RND_OM: which product of om f + w h is rounded first (om f, else w h).
-template <class W, bool SHIFT, bool RND_OM>
+// RI, RO: which product of om f + w h is rounded first, om f or (false) w h, for
+// fi and fo.
+template <class W, bool SHIFT, bool RI, bool RO>
 __device__ __forceinline__ void relax_pair(W& fi, W& fo, W e, typename Vec<W>::A w, W nusq, W R, W R3, W nR3, W B, W om,
                                            W nomega) {
     typedef Vec<W> K;
@@ -591,8 +555,8 @@ __device__ __forceinline__ void relax_pair(W& fi, W& fo, W e, typename Vec<W>::A
     const W h = vfma(R, q, B);
     const W hp = vfma(R3, e, h), hm = vfma(nR3, e, h);
     if (SHIFT) {
-        fi = RND_OM ? vfma(K::all(w), hp, vmul(om, fi)) : vfma(om, fi, vmul(K::all(w), hp));
-        fo = RND_OM ? vfma(K::all(w), hm, vmul(om, fo)) : vfma(om, fo, vmul(K::all(w), hm));
+        fi = RI ? vfma(K::all(w), hp, vmul(om, fi)) : vfma(om, fi, vmul(K::all(w), hp));
+        fo = RO ? vfma(K::all(w), hm, vmul(om, fo)) : vfma(om, fo, vmul(K::all(w), hm));
     } else {  // here R = rho, R3 = 3 rho, B = rho
         fi = vfma(nomega, vfma(K::all(-w), hp, fi), fi);
         fo = vfma(nomega, vfma(K::all(-w), hm, fo), fo);
@@ -606,14 +570,48 @@ __device__ __forceinline__ bool rho_ok(double rho) {
     return (unsigned long long)__double_as_longlong(rho) - 1ull < 0x46293E5939A08CEAull - 1ull;  // 1e30
 }
 
+// The strain A = 3 sqrt|Pi_xy^2 - Pi_xx Pi_yy| / rho of the nodes of W, from
+// populations as collide_nodes takes them.
+template <class W, bool SHIFT, bool SC>
+__device__ __forceinline__ W strain(const W (&f)[9], const HotPrm<typename Vec<W>::A>& H) {
+    typedef Vec<W> K;
+    typedef typename K::A A;
+    const W a = vadd(vadd(f[1], f[5]), f[8]), b = vadd(vadd(f[3], f[6]), f[7]);
+    const W c = vadd(vadd(f[2], f[5]), f[6]), d = vadd(vadd(f[4], f[7]), f[8]);
+    W s = vadd(vadd(f[0], vadd(f[2], f[4])), vadd(a, b)), jx = vsub(a, b), jy = vsub(c, d);
+    W ab = vadd(a, b), cd = vadd(c, d), sxy = vsub(vadd(f[5], f[7]), vadd(f[6], f[8]));
+    if (SC) {  // unscaled
+        const W u1 = K::all(H.inv_scale);
+        s = vmul(s, u1);
+        jx = vmul(jx, u1);
+        jy = vmul(jy, u1);
+        ab = vmul(ab, u1);
+        cd = vmul(cd, u1);
+        sxy = vmul(sxy, u1);
+    }
+    const W rho = SHIFT ? vadd(K::all(H.rho0), s) : s;
+    W irho, r;
+#pragma unroll
+    for (int k = 0; k < K::N; ++k) K::set(irho, k, rcp_rho<A>(K::get(rho, k)));
+    const W njr = vmul(irho, K::all((A)-1)), third = K::all((A)(-1.0 / 3.0));  // s: rho, or rho - rho0 of shifted values
+    const W pxx = vfma(vmul(jx, jx), njr, vfma(s, third, ab));
+    const W pyy = vfma(vmul(jy, jy), njr, vfma(s, third, cd));
+    const W pxy = vfma(vmul(jx, jy), njr, sxy);
+    const W det = vfma(pxy, pxy, vmul(vmul(K::all((A)-1), pxx), pyy));
+#pragma unroll
+    for (int k = 0; k < K::N; ++k) K::set(r, k, (A)3 * sqrt(fabs(K::get(det, k))) * K::get(irho, k));
+    return r;
+}
+
 // SC (shifted stores only): f holds (f - w_i rho0) * s in the store's scaled
 // units, s = H.scale, and so does the result; the moments are unscaled once
 // per node (exact: s is a power of two) instead of every population.  The
-// components of W are nodes, th their normals (NOISE and X.kT > 0: thetas());
-// returns their densities.
+// components of W are nodes, th their normals (NOISE and X.kT > 0: thetas()),
+// tau their relaxation times (PL: solve_taus() of strain()); returns their
+// densities.
 template <class W, bool SHIFT, bool NOISE, bool PL, bool SC = false>
 __device__ __forceinline__ W collide_nodes(W (&f)[9], const HotPrm<typename Vec<W>::A>& H,
-                                           const ExtPrm<typename Vec<W>::A>& X, const W (&th)[6]) {
+                                           const ExtPrm<typename Vec<W>::A>& X, const W (&th)[6], W tau) {
     static_assert(!SC || SHIFT, "scaled units are those of the shifted stores");
     typedef Vec<W> K;
     typedef typename K::A A;
@@ -633,30 +631,8 @@ __device__ __forceinline__ W collide_nodes(W (&f)[9], const HotPrm<typename Vec<
     for (int k = 0; k < K::N; ++k) K::set(irho, k, rcp_rho<A>(K::get(rho, k)));
     W omega = K::all(H.omega), om = K::all(H.om), tgx = K::all(H.tgx), tgy = K::all(H.tgy);
     if (PL) {
-        const W drho = SHIFT ? s : vsub(s, K::all(H.rho0));
-        const W d3 = SHIFT ? drho : rho;  // 3 x the isotropic part
-        W ab = vadd(a, b), cd = vadd(c, d), sxy = vsub(vadd(f[5], f[7]), vadd(f[6], f[8]));
-        if (SC) { ab = vmul(ab, u1); cd = vmul(cd, u1); sxy = vmul(sxy, u1); }  // unscaled second moments
-        const W njr = vmul(irho, K::all((A)-1));
-        const W pxx = vfma(vmul(jx, jx), njr, vfma(d3, K::all((A)(-1.0 / 3.0)), ab));
-        const W pyy = vfma(vmul(jy, jy), njr, vfma(d3, K::all((A)(-1.0 / 3.0)), cd));
-        const W pxy = vfma(vmul(jx, jy), njr, sxy);
-        const W det = vfma(pxy, pxy, vmul(vmul(K::all((A)-1), pxx), pyy));
-        // A = 3 sqrt|det| / rho
-        W root;
-        if constexpr (sizeof(A) == 8) {
-            root = sqrt(fabs(det));
-        } else {
-            root = sqrt_hw(vabs(det));
-        }
-        const W tau = solve_taus(vmul(vmul(K::all((A)3), root), irho), X);
-        if constexpr (sizeof(A) == 8) {
-            omega = 1.0 / tau;
-        } else {  // the reciprocal and one Newton step
 #pragma unroll
-            for (int k = 0; k < K::N; ++k) K::set(omega, k, rcp_rho<float>(K::get(tau, k)));
-            omega = vfma(vfma(vmul(K::all((A)-1), tau), omega, K::all((A)1)), omega, omega);
-        }
+        for (int k = 0; k < K::N; ++k) K::set(omega, k, (A)1 / K::get(tau, k));
         om = vsub(K::all((A)1), omega);
         tgx = vmul(tau, K::all(X.gx));
         tgy = vmul(tau, K::all(X.gy));
@@ -670,16 +646,15 @@ __device__ __forceinline__ W collide_nodes(W (&f)[9], const HotPrm<typename Vec<
     const W R3 = vmul(K::all((A)3), R), nR3 = vmul(K::all((A)-3), R);
     const W nomega = vmul(K::all((A)-1), omega);
     const W h0 = vfma(R, nusq, B);
-    if (SHIFT && PL) f[0] = vfma(K::all((A)wgt(0)), h0, vmul(om, f[0]));
-    else if (SHIFT) f[0] = vfma(om, f[0], vmul(K::all((A)wgt(0)), h0));
+    if (SHIFT) f[0] = vfma(om, f[0], vmul(K::all((A)wgt(0)), h0));
     else f[0] = vfma(nomega, vfma(K::all(-(A)wgt(0)), h0, f[0]), f[0]);
-    relax_pair<W, SHIFT, PL>(f[1], f[3], ux, (A)wgt(1), nusq, R, R3, nR3, B, om, nomega);
-    relax_pair<W, SHIFT, PL>(f[2], f[4], uy, (A)wgt(2), nusq, R, R3, nR3, B, om, nomega);
-    relax_pair<W, SHIFT, PL>(f[5], f[7], vadd(ux, uy), (A)wgt(5), nusq, R, R3, nR3, B, om, nomega);
-    // (the half-precision stores turn any other rounding into differences of an
-    // ulp of theirs, so the last pair keeps the order it always had; with the
-    // power law tau* often sits at its upper clamp 2, where om f is exact)
-    relax_pair<W, SHIFT, !NOISE || PL>(f[6], f[8], vsub(uy, ux), (A)wgt(6), nusq, R, R3, nR3, B, om, nomega);
+    relax_pair<W, SHIFT, false, false>(f[1], f[3], ux, (A)wgt(1), nusq, R, R3, nR3, B, om, nomega);
+    relax_pair<W, SHIFT, false, false>(f[2], f[4], uy, (A)wgt(2), nusq, R, R3, nR3, B, om, nomega);
+    relax_pair<W, SHIFT, false, PL>(f[5], f[7], vadd(ux, uy), (A)wgt(5), nusq, R, R3, nR3, B, om, nomega);
+    // The orders of the roundings are those the code had before it was packed:
+    // the half-precision stores turn any other into differences of an ulp of
+    // theirs, and tau* of shear-thinning fluids amplifies those of the strain.
+    relax_pair<W, SHIFT, !NOISE || PL, !NOISE || PL>(f[6], f[8], vsub(uy, ux), (A)wgt(6), nusq, R, R3, nR3, B, om, nomega);
     if (NOISE) {
         if (X.kT > (A)0) {
             W amp;

@@ -278,13 +278,32 @@ __device__ __forceinline__ bool finish_chunk(const StreamArgs& a, const DomDev& 
             }
         }
     }
+    W tau[ChunkOf<S>::N];
+    if constexpr (PL) {
+        typename S::A as[V], ts[V];
+#pragma unroll
+        for (int p = 0; p < ChunkOf<S>::N; ++p) {
+            W n9[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) n9[i] = f[i][p];
+            const W r = strain<W, S::SHIFT, S::SCALED>(n9, H);
+#pragma unroll
+            for (int k = 0; k < N; ++k) as[p * N + k] = K::get(r, k);
+        }
+        solve_taus(as, X, ts);
+#pragma unroll
+        for (int k = 0; k < V; ++k) K::set(tau[k / N], k % N, ts[k]);
+    } else {
+#pragma unroll
+        for (int p = 0; p < ChunkOf<S>::N; ++p) tau[p] = K::all(0);
+    }
     if (!fix)
 #pragma unroll
     for (int p = 0; p < ChunkOf<S>::N; ++p) {
         W n9[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) n9[i] = f[i][p];
-        const W rho = collide_nodes<W, S::SHIFT, NOISE, PL, S::SCALED>(n9, H, X, th[p]);
+        const W rho = collide_nodes<W, S::SHIFT, NOISE, PL, S::SCALED>(n9, H, X, th[p], tau[p]);
 #pragma unroll
         for (int k = 0; k < N; ++k)
             if (rho_ok(K::get(rho, k))) good |= 1u << (p * N + k);
