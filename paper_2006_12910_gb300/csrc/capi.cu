@@ -65,7 +65,7 @@ struct lbm_ctx {
     std::vector<DomDev> hd;
     std::vector<std::vector<uint8_t>> hsolid;  // host copy of each domain's mask (ny*nx)
     DomDev* dd = nullptr;
-    int64_t* d_item_off = nullptr;
+    uint16_t* item_dom = nullptr;        // [total_items], several domains only
     int64_t total_items = 0;
     void* f[2] = {nullptr, nullptr};
     size_t arena_elems = 0;
@@ -438,7 +438,7 @@ cudaError_t enqueue_stream_collide(lbm_ctx* c, int cur, cudaStream_t s, int bloc
                                    int mode = STREAM_ALL, bool with_flips = true, bool pdl = false) {
     StreamArgs a;
     a.doms = c->dd;
-    a.item_off = c->d_item_off;
+    a.item_dom = c->item_dom;
     a.ndom = c->ndom;
     a.total_items = c->total_items;
     a.src = c->f[cur];
@@ -719,7 +719,7 @@ int lbm_create_ensemble(int ndom, const lbm_params* per_domain, void* cuda_strea
     c->prm.assign(per_domain, per_domain + ndom);
     c->hd.resize(ndom);
     c->hsolid.resize(ndom);
-    std::vector<int64_t> item_off(ndom);
+    std::vector<uint16_t> item_dom;
     int64_t off = 0, node_off = 0, mask_off = 0, items = 0;
     int pslot = 0;
     for (int d = 0; d < ndom; ++d) {
@@ -731,7 +731,7 @@ int lbm_create_ensemble(int ndom, const lbm_params* per_domain, void* cuda_strea
         D.item_off = items;
         D.p0 = pslot;
         D.np = 0;
-        item_off[d] = items;
+        if (ndom > 1) item_dom.insert(item_dom.end(), (size_t)D.ny * D.seg_per_row, (uint16_t)d);
         off += 9 * D.plane;
         node_off += D.plane;
         mask_off += (int64_t)D.ny * D.seg_per_row;
@@ -839,7 +839,7 @@ int lbm_create_ensemble(int ndom, const lbm_params* per_domain, void* cuda_strea
         }
     }
     CKCR(dev_malloc(&c->dd, sizeof(DomDev) * ndom));
-    CKCR(dev_malloc(&c->d_item_off, sizeof(int64_t) * ndom));
+    if (ndom > 1) CKCR(dev_malloc(&c->item_dom, sizeof(uint16_t) * item_dom.size()));
     CKCR(dev_malloc(&c->ctr, sizeof(int64_t) * 2));
     CKCR(dev_malloc(&c->pstep, sizeof(int64_t) * 2));
     CKCR(cudaMemsetAsync(c->pstep, 0, sizeof(int64_t) * 2, c->stream));
@@ -852,7 +852,8 @@ int lbm_create_ensemble(int ndom, const lbm_params* per_domain, void* cuda_strea
     CKCR(cudaMemsetAsync(c->ctr, 0, sizeof(int64_t) * 2, c->stream));
     CKCR(cudaMemsetAsync(c->err, 0, sizeof(unsigned), c->stream));
     CKCR(cudaMemcpyAsync(c->dd, c->hd.data(), sizeof(DomDev) * ndom, cudaMemcpyHostToDevice, c->stream));
-    CKCR(cudaMemcpyAsync(c->d_item_off, item_off.data(), sizeof(int64_t) * ndom, cudaMemcpyHostToDevice, c->stream));
+    if (ndom > 1)
+        CKCR(cudaMemcpyAsync(c->item_dom, item_dom.data(), sizeof(uint16_t) * item_dom.size(), cudaMemcpyHostToDevice, c->stream));
     CKCR(cudaStreamSynchronize(c->stream));
     for (int d = 0; d < ndom; ++d)
         if ((r = upload_geometry(c, d)) != LBM_OK) { g_create_error = c->msg; return cleanup(r); }
@@ -881,7 +882,7 @@ void lbm_destroy(lbm_ctx* c) {
         for (auto& g : gk)
             if (g) cudaGraphExecDestroy(g);
     cudaFree(c->f[0]); cudaFree(c->f[1]); cudaFree(c->solid); cudaFree(c->nflags); cudaFree(c->special);
-    cudaFree(c->dd); cudaFree(c->d_item_off); cudaFree(c->ctr); cudaFree(c->pstep); cudaFree(c->err);
+    cudaFree(c->dd); cudaFree(c->item_dom); cudaFree(c->ctr); cudaFree(c->pstep); cudaFree(c->err);
     cudaFree(c->d_partial); cudaFree(c->d_sums); cudaFree(c->d_stage); cudaFree(c->d_mom);
     if (c->h_mom) cudaFreeHost(c->h_mom);
     if (c->h_pin) cudaFreeHost(c->h_pin);

@@ -134,25 +134,40 @@ __global__ void k_moments(DomDev D, const typename S::T* arena, const uint8_t* s
 // numbers, each addition error-free (Knuth's TwoSum, The Art of Computer
 // Programming vol. 2, Sec. 4.2.2): 14 TwoSums a node, about 48 bits, so that
 // the rounding to the FP32 output is the same as from FP64 sums.
-struct FF {
-    float h, l;
+// FP32 stores carry two nodes in the packed instructions.
+template <class W>
+struct FFW {
+    W h, l;
 };
+typedef FFW<float> FF;
 struct MomPrm {  // rho0 and g / 2 as pairs, split on the host; FP64 store: its fixed-point format (e0 0: none)
     FF rho0, gx2, gy2;
     int32_t e0;
     float unit;
 };
-__device__ __forceinline__ FF two_sum(float a, float b) {
-    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
-    return FF{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+template <class W>
+__device__ __forceinline__ FFW<W> two_sum(W a, W b) {
+    const W s = vadd(a, b), bb = vsub(s, a);
+    return FFW<W>{s, vadd(vsub(a, vsub(s, bb)), vsub(b, bb))};
 }
-__device__ __forceinline__ FF add(FF a, float b) {
-    const FF s = two_sum(a.h, b);
-    return FF{s.h, __fadd_rn(s.l, a.l)};
+template <class W>
+__device__ __forceinline__ FFW<W> add(FFW<W> a, W b) {
+    const FFW<W> s = two_sum(a.h, b);
+    return FFW<W>{s.h, vadd(s.l, a.l)};
 }
-__device__ __forceinline__ FF add(FF a, FF b) {
-    const FF s = two_sum(a.h, b.h);
-    return FF{s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l))};
+template <class W>
+__device__ __forceinline__ FFW<W> add(FFW<W> a, FFW<W> b) {
+    const FFW<W> s = two_sum(a.h, b.h);
+    return FFW<W>{s.h, vadd(s.l, vadd(a.l, b.l))};
+}
+template <class W>
+__device__ __forceinline__ FFW<W> sub(FFW<W> a, FFW<W> b) {
+    const W m = Vec<W>::all(-1.0f);
+    return add(a, FFW<W>{vmul(b.h, m), vmul(b.l, m)});
+}
+template <class W>
+__device__ __forceinline__ FFW<W> all(FF x) {
+    return FFW<W>{Vec<W>::all(x.h), Vec<W>::all(x.l)};
 }
 // A number of units of the fixed-point format as a pair.
 __device__ __forceinline__ FF pair_of(int64_t x) {
@@ -163,11 +178,13 @@ __device__ __forceinline__ FF pair_of(int64_t x) {
 }
 // j / r - g2 (the velocity (j - r g / 2) / r) from the pairs, y about 1 / r:
 // the quotient's first digit and the remainder's, then the body-force term.
-__device__ __forceinline__ float velocity(FF j, FF r, float y, FF g2) {
-    const float q = __fmul_rn(j.h, y);
-    const float rem = __fadd_rn(__fmaf_rn(-q, r.h, j.h), __fmaf_rn(-q, r.l, j.l));
-    const FF u = two_sum(q, -g2.h);
-    return __fadd_rn(u.h, __fadd_rn(u.l, __fmaf_rn(rem, y, -g2.l)));
+template <class W>
+__device__ __forceinline__ W velocity(FFW<W> j, FFW<W> r, W y, FF g2) {
+    typedef Vec<W> K;
+    const W q = vmul(j.h, y), nq = vmul(q, K::all(-1.0f));
+    const W rem = vadd(vfma(nq, r.h, j.h), vfma(nq, r.l, j.l));
+    const FFW<W> u = two_sum(q, K::all(-g2.h));
+    return vadd(u.h, vadd(u.l, vfma(rem, y, K::all(-g2.l))));
 }
 
 // One chunk of V = 4 nodes (FP64 store: 2) a thread: one vector load per plane,
@@ -197,45 +214,65 @@ __global__ void __launch_bounds__(256) k_moments_f32(const __grid_constant__ Dom
     const int y = (int)(k / chunks), x0 = (int)(k - (uint32_t)y * chunks) * V;
     const int64_t ni = (int64_t)y * D.pitch + x0, o = (int64_t)y * D.nx + x0;
     const typename S::T* p = arena + D.off + ni;
-    A f[9][V];
+    // nodes in vectors W: FP32 stores two at a time
+    typedef typename ChunkOf<S>::W W;
+    typedef Vec<W> K;
+    constexpr int N = K::N;
+    W f[9][V / N];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) load_vec<S, V>(p + (int64_t)i * D.plane, f[i], sizeof(A) == 4 ? (A)D.inv_scale_f : (A)1);
+    for (int i = 0; i < 9; ++i) {
+        A v[V];
+        load_vec<S, V>(p + (int64_t)i * D.plane, v, sizeof(A) == 4 ? (A)D.inv_scale_f : (A)1);
+#pragma unroll
+        for (int k = 0; k < V; ++k) K::set(f[i][k / N], k % N, v[k]);
+    }
     uint8_t sol[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) sol[v] = solid[D.node_off + ni + v];
     float rho[V], ux[V], uy[V];
+    bool plain[V];
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-        bool plain;
+    for (int m = 0; m < V / N; ++m) {
         if constexpr (sizeof(A) == 8) {
             // FP64 store: exact sums in the fixed-point format of the collision
             uint32_t t = 0;
             int64_t g[9];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) g[i] = to_fix(f[i][v], P.e0, t);
+            for (int i = 0; i < 9; ++i) g[i] = to_fix(f[i][m], P.e0, t);
             const int64_t a = g[1] + g[5] + g[8], b = g[3] + g[6] + g[7];
             const int64_t c = g[2] + g[5] + g[6], d = g[4] + g[7] + g[8];
             const FF r = pair_of(g[0] + g[2] + g[4] + a + b);
             const float rs = __fadd_rn(r.h, r.l), yr = rcp_rho<float>(rs);
-            rho[v] = rs * P.unit;
-            plain = P.e0 != 0 && t < FIX_RANGE && rho[v] > 1e-30f && rho[v] < 1e30f;
-            ux[v] = velocity(pair_of(a - b), r, yr, P.gx2);
-            uy[v] = velocity(pair_of(c - d), r, yr, P.gy2);
+            rho[m] = rs * P.unit;
+            plain[m] = P.e0 != 0 && t < FIX_RANGE && rho[m] > 1e-30f && rho[m] < 1e30f;
+            ux[m] = velocity<float>(pair_of(a - b), r, yr, P.gx2);
+            uy[m] = velocity<float>(pair_of(c - d), r, yr, P.gy2);
         } else {
-            const FF a = add(two_sum(f[5][v], f[8][v]), f[1][v]), b = add(two_sum(f[6][v], f[7][v]), f[3][v]);
-            const FF c = add(two_sum(f[5][v], f[6][v]), f[2][v]), d = add(two_sum(f[7][v], f[8][v]), f[4][v]);
-            FF r = add(add(two_sum(f[2][v], f[4][v]), f[0][v]), add(a, b));
-            if (S::SHIFT) r = add(P.rho0, r);
-            const FF jx = add(a, FF{-b.h, -b.l}), jy = add(c, FF{-d.h, -d.l});
-            rho[v] = __fadd_rn(r.h, r.l);
-            plain = rho[v] > 1e-30f && rho[v] < 1e30f;
-            const float yr = rcp_rho<float>(rho[v]);
-            ux[v] = velocity(jx, r, yr, P.gx2);
-            uy[v] = velocity(jy, r, yr, P.gy2);
+            const FFW<W> a = add(two_sum(f[5][m], f[8][m]), f[1][m]), b = add(two_sum(f[6][m], f[7][m]), f[3][m]);
+            const FFW<W> c = add(two_sum(f[5][m], f[6][m]), f[2][m]), d = add(two_sum(f[7][m], f[8][m]), f[4][m]);
+            FFW<W> r = add(add(two_sum(f[2][m], f[4][m]), f[0][m]), add(a, b));
+            if (S::SHIFT) r = add(all<W>(P.rho0), r);
+            const W rs = vadd(r.h, r.l);
+            W yr;
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                rho[m * N + k] = K::get(rs, k);
+                plain[m * N + k] = K::get(rs, k) > 1e-30f && K::get(rs, k) < 1e30f;
+                K::set(yr, k, rcp_rho<float>(K::get(rs, k)));
+            }
+            const W vx = velocity(sub(a, b), r, yr, P.gx2), vy = velocity(sub(c, d), r, yr, P.gy2);
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                ux[m * N + k] = K::get(vx, k);
+                uy[m * N + k] = K::get(vy, k);
+            }
         }
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
         if (sol[v]) {
             rho[v] = ux[v] = uy[v] = 0.0f;
-        } else if (!plain && x0 + v < D.nx) {  // not finite, not positive or out of range: as the FP64 sums give it
+        } else if (!plain[v] && x0 + v < D.nx) {  // not finite, not positive or out of range: as the FP64 sums give it
             double r, u0, u1;
             node_moments_f64<S>(D, arena, ni + v, r, u0, u1);
             rho[v] = (float)r;

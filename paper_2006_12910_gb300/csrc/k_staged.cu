@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(STAGED_MAX_BLOCK) k_stream_staged(StreamArgs a
         int near = 0, d = 0, y = 0, seg = 0, spec = 0;
         if (valid) {
             near = __ldg(a.mark + (int64_t)par * a.total_items + g) == (int32_t)step64;
-            d = a.ndom == 1 ? 0 : find_domain(a.item_off, a.ndom, g);
+            d = a.ndom == 1 ? 0 : (int)__ldg(a.item_dom + g);
             const Geo G = load_geo(a.doms[d]);
             const int local = (int)(g - G.item_off);
             y = local / G.spr;

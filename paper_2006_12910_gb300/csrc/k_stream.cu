@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(REG_K1_MAX_BLOCK, (k1_min_blocks<S, NOISE, PL>
         if (a.mode == STREAM_NEAR)
             g = __shfl_sync(0xffffffffu, (uint32_t)__ldg(a.near_list + (int64_t)par * a.total_items + w), 0);
         else if (a.mode == STREAM_FAR || FLIPS) mk = __ldg(mark + w);
-        const int d = one ? 0 : __shfl_sync(0xffffffffu, find_domain(a.item_off, a.ndom, g), 0);
+        const int d = one ? 0 : (int)__ldg(a.item_dom + g);
         const DomDev& D = a.doms[d];
         const Geo G = one ? param_geo(a.dom0) : load_geo(D);
         const int nx = G.nx;

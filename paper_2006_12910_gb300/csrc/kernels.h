@@ -11,7 +11,7 @@ namespace lbmk {
 struct StreamArgs {
     DomDev dom0;              // copy of doms[0] in the launch parameters (read when ndom == 1)
     const DomDev* doms;
-    const int64_t* item_off;  // first work item of each domain (ndom entries)
+    const uint16_t* item_dom; // domain of each work item (ndom > 1)
     int ndom;
     int64_t total_items;      // sum over domains of ny * seg_per_row
     const void* src;          // population arena holding f*(t) (after link swaps)

@@ -13,15 +13,6 @@
 
 namespace lbmk {
 
-__device__ __forceinline__ int find_domain(const int64_t* __restrict__ item_off, int ndom, int64_t g) {
-    int lo = 0, hi = ndom - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(item_off + mid) <= g) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
 // Geometry of one domain for a work item, read with 16-byte loads.
 struct Geo {
     int nx, ny, pitch, flags;
