@@ -1,13 +1,15 @@
 // capi.cu -- host runtime and C ABI of the GB300 D2Q9 library (include/lbm.h).
 //
 // The context owns every device buffer: two population arenas (the state
-// f*(t) and the next state), per-node solid bytes, the per-chunk slow-path
-// bitmask, the step counters, a sticky error word and the particle arrays.
+// f*(t) and the next state), per-node solid bytes and flag words, the per-chunk
+// flag bits, the step counters, a sticky error word and the particle arrays.
 // lbm_step replays CUDA graphs of 2^j timesteps, j = 0 .. GRAPH_LOG (the
-// binary digits of the step count, largest first); a timestep is
-//   [particle forces + Newton-Euler] -> [link exchange + re-rasterise]
-//   -> [fused pull-stream + collide over every domain]
-// where the two particle kernels are skipped when no domain holds particles.
+// binary digits of the step count, largest first), each built when a call first
+// needs it, or one graph of a count that lbm_prepare_steps prepared; a timestep is
+//   [particle forces + Newton-Euler + link exchange]
+//   -> [fused pull-stream + collide over every domain], beside it
+//   [re-rasterise, Eq. MP2 sums for later steps]
+// where the particle kernels are skipped when no domain holds particles.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -443,7 +445,6 @@ cudaError_t enqueue_stream_collide(lbm_ctx* c, int cur, cudaStream_t s, int bloc
     a.total_items = c->total_items;
     a.src = c->f[cur];
     a.dst = c->f[cur ^ 1];
-    a.solid = c->solid;
     a.nflags = c->nflags;
     a.special = c->special;
     a.ctr_in = c->ctr + cur;

@@ -4,21 +4,23 @@
 //
 // Same work items as k_stream.cu (one item = one domain row segment of
 // 32 * V nodes), but nothing of an item passes through registers before it
-// is needed.  One lane of the warp issues nine cp.async.bulk copies (one per
-// direction plane, from the row that direction pulls from) and, for segments
-// with flagged nodes, one copy of the flag words, into a shared-memory stage,
-// and arms the stage's mbarrier with the expected byte count; each warp keeps
+// is needed.  Lane 0 arms the stage's mbarrier with the expected byte count;
+// lanes 0-8 issue one cp.async.bulk copy each (one per direction plane, from
+// the row that direction pulls from), lanes 9-14 the blocks with the wrapped
+// elements of periodic row ends and, for segments with flagged nodes, lane 15
+// that of the flag words, into a shared-memory stage; each warp keeps
 // `stages` items in flight and computes the oldest while the others stream
 // in, so the bytes in flight per SM are set by shared memory, not registers.
 //
 // A stage holds, per plane, the segment plus one 16-byte halo on each side:
 // element j of a plane row is x = xs - E + j (xs the segment's first node,
 // E = 16 / sizeof(T)), clipped to [0, pitch) at the row ends.  Lane l then
-// takes nodes xs + l + 32 k one at a time: the nine pulled values are plain
-// shared-memory reads at x - e_ix, so only one node's populations are live in
-// registers, and every store of the warp writes 32 consecutive elements.
-// Only nodes at x = 0 or nx - 1 read a wrapped source from global memory
-// (periodic x) or take the Zou-He / corner patch (open ends).  Every mbarrier
+// reads its chunk of V nodes and the edge elements from shared memory and goes
+// on as the register kernel does (form_chunk, patch_chunk, finish_chunk; equal
+// results).  The register kernel is the default: a bulk copy costs its SM about
+// 40 cycles here, and nine small ones an item (1 KB a row at most) made this
+// kernel 30 us against 26.5 (FP32, 2048x1024) and 20.6 against 14.4 (FP16).
+// Open ends and corners read their sources from global memory.  Every mbarrier
 // wait is bounded (about one second by the global timer); a wait that runs
 // out sets ERR_TIMEOUT, waits (bounded again, always by the full second) for
 // the warp's copies in flight and ends the warp's work.  The limit of the

@@ -79,8 +79,8 @@ struct alignas(16) DomDev {
 // Per-node flag words (uint16), written from the geometry on the host.  Bit j
 // (1..8): the neighbour x + e_j of a fluid node is solid or lies beyond a y
 // wall, and the node pulls its population opp(j) from its own slot j instead
-// (halfway bounce-back).  A chunk whose nodes all have zero flags takes the
-// plain vector path without reading them.
+// (halfway bounce-back).  The stream-collide kernels load the words of every
+// chunk with its populations (the staged kernel those of flagged segments).
 enum : uint16_t {
     NF_SOLID = 1u << 0,
     NF_ZH_IN = 1u << 9,    // Zou-He inlet node (x = 0)
