@@ -675,6 +675,22 @@ def main():
                 # the whole step against the same bound: fluid-node updates per second x bytes per update
                 "step_frac": fluid * args.steps / (ms * 1e-3) * 2 * 9 * S / 1e9 / peak}
 
+    # The same pass as the steps of a graph: the workload without its particles, whose step is
+    # one pass over every item (plain launches back to back are spaced by the launch path).
+    pf = lbm.Context(lbm.make_params(nx=w.nx, ny=w.ny, store=args.store, store_scale=scale, **base),
+                     stream=stream.cuda_stream, solids=[w.solid])
+    pf.set_launch(*launch[:3])
+    pf.prepare_steps(n_ts)
+    pf.step(n_ts)
+    pf.sync()
+    e0.record(stream)
+    pf.step(n_ts)
+    e1.record(stream)
+    e1.synchronize()
+    pf.close()
+    pg = e0.elapsed_time(e1) / n_ts
+    roofline.update(kernel_ms_in_graph=pg, frac_in_graph=alg_bytes / (pg * 1e-3) / 1e9 / peak)
+
     # ---- end to end through the C ABI with host buffers ------------------------------------
     # Upload the initial state from pinned host memory, then every step: advance and read
     # the particle state back to the host; finally read the moment fields back.

@@ -287,9 +287,9 @@ int lbm_profile_steps(lbm_ctx* ctx, int64_t nsteps, double* ms_out3, int64_t* la
  * Blocking.  LBM_E_INVAL for nlaunches < 1 or ms_out NULL. */
 int lbm_time_stream(lbm_ctx* ctx, int32_t nlaunches, double* ms_out);
 
-/* Measurement of the device's FP64 rate (no paper counterpart; it sets the
- * arithmetic roofline of the FP64 store, whose collision is bound by FP64
- * issue on this part rather than by HBM).  Eight independent FMA chains in
+/* Measurement of the device's FP64 rate (no paper counterpart; it bounds the
+ * FP64 store with noise or the power law; its plain collision is computed in
+ * 64-bit fixed point, because FP64 issue is slow on this part).  Eight independent FMA chains in
  * every thread of 8 CTAs x 256 threads per SM, timed with CUDA events on
  * cuda_stream (NULL: the default stream), best of three launches after one
  * warm-up; *gflops_out = 2 x FMAs / second / 1e9.  Blocking; allocates

@@ -194,10 +194,10 @@ __device__ __forceinline__ W velocity(FFW<W> j, FFW<W> r, W y, FF g2) {
 // another without the launch gap; each still waits for the one before it.
 // Bound by HBM (FP32 stores: 70 % of the copy rate) and, for the half-precision
 // stores, by arithmetic.  Measured, launches back to back, against FP64
-// sums and divisions a node at a time: 2048x1024 shifted FP32 260 -> 20.9 us,
-// FP16 265 -> 17.3, FP64 191 -> 33 (exact sums in the fixed-point
-// format of the collision); 96 ensemble domains (96 launches) 1812 -> 344;
-// 4096x2048 1023 -> 77.
+// sums and divisions a node at a time: 2048x1024 shifted FP32 260 -> 18.2 us,
+// FP16 265 -> 13.5, FP64 191 -> 33 (exact sums in the fixed-point
+// format of the collision); 96 ensemble domains (96 launches) 1812 -> 344 or
+// less; 4096x2048 1023 -> 72.
 template <class S>
 __host__ __device__ constexpr int moment_chunk() { return sizeof(typename S::T) == 8 ? 2 : 4; }
 template <class S, bool ALIGNED>
