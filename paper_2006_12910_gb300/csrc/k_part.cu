@@ -1179,13 +1179,21 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(c
             const int r = r0 + lane;
             int y = y0 + r, xdummy = 0;
             const bool row_ok = r < nrows && wrap_node(D, xdummy, y);
-            for (int xx = x0;; xx += seg_w) {
-                const int xc = xx < x1 ? xx : x1;
-                int x = xc, yd = 0;
+            // one node of every item of the range: from item to item, the last one
+            // of a row shorter than the others
+            for (int xx = x0; xx <= x1;) {
+                int x = xx, yd = 0;
+                if (!wrap_node(D, x, yd)) {  // beyond an open end
+                    if (xx >= D.nx) break;
+                    xx = 0;
+                    continue;
+                }
+                const int seg = x / seg_w;
+                xx += min((seg + 1) * seg_w, D.nx) - x;
                 bool need = false;
                 int64_t item = 0;
-                if (row_ok && wrap_node(D, x, yd)) {
-                    item = D.item_off + (int64_t)y * D.seg_per_row + x / seg_w;
+                if (row_ok) {
+                    item = D.item_off + (int64_t)y * D.seg_per_row + seg;
                     int32_t* m = a.mark + (int64_t)mpar * a.total_items + item;
                     need = atomicExch(m, (int32_t)t_next) != (int32_t)t_next;
                 }
@@ -1198,7 +1206,6 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(c
                         a.near_list[(int64_t)lpar * a.total_items + base + __popc(bal & ((1u << lane) - 1u))] =
                             (int32_t)item;
                 }
-                if (xc == x1) break;
             }
         }
         return;
