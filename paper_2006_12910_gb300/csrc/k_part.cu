@@ -1162,13 +1162,21 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(c
     const int wpar = (int)(t_next & 1);
     if (HI >= 3 && role == 3) {
         // ------------------------------------------------------------------ role C
-        // Work items (row segments) within two nodes of the disk's boxes at t
-        // and t+1 are "near": the stream-collide pass of that step runs them
-        // after this kernel, and they hold every node that changes side.
+        // Work items (row segments) within two rows, and mx nodes of a row, of the
+        // disk's boxes at t and t+1 are "near": the stream-collide pass of that
+        // step runs them after this kernel, and they hold every node that
+        // changes side.  mx is what the staged kernel copies beyond a segment
+        // (16 bytes): a FAR pass runs beside the link exchange and reads none of
+        // the slots that it rewrites.
+        constexpr int mx = 16 / (int)sizeof(typename S::T);
         const int mpar = (int)(t_next % 3);  // three-way: the passes of t and t+1 read the other two
         const int lpar = (int)(t_next % 3);
         const Box bo = uni.bo, bn = uni.bn;
-        const int x0 = min(bo.x0, bn.x0) - 2, x1 = max(bo.x0 + bo.w, bn.x0 + bn.w) + 1;
+        int x0 = min(bo.x0, bn.x0) - mx, x1 = max(bo.x0 + bo.w, bn.x0 + bn.w) + mx - 1;
+        if (px && x1 - x0 >= D.nx) {  // once around: every item of the rows
+            x0 = 0;
+            x1 = D.nx - 1;
+        }
         const int y0 = min(bo.y0, bn.y0) - 2, y1 = max(bo.y0 + bo.h, bn.y0 + bn.h) + 1;
         const int seg_w = 32 * D.V;
         const int lane = threadIdx.x & 31;

@@ -62,14 +62,26 @@ __global__ void __launch_bounds__(REG_K1_MAX_BLOCK, (k1_min_blocks<S, NOISE, PL>
     const uint32_t count = a.mode == STREAM_NEAR ? (uint32_t)__ldg(a.near_cnt + par) : (uint32_t)a.total_items;
     const int32_t next_stamp = (int32_t)(step64 + 1);
     const int32_t* mark = a.mark + (int64_t)par * a.total_items;
-    const bool one = a.ndom == 1;
+    const bool one = a.ndom == 1, far = a.mode == STREAM_FAR;
 
-    for (uint32_t w = blockIdx.x * wpb + warp; w < count; w += nwarps) {
+    uint32_t w = blockIdx.x * wpb + warp;
+    int32_t mk_next = far && w < count ? __ldg(mark + w) : 0;
+    for (; w < count; w += nwarps) {
         uint32_t g = w;
         int32_t mk = (int32_t)step64;
-        if (a.mode == STREAM_NEAR)
+        if (a.mode == STREAM_NEAR) {
             g = __shfl_sync(0xffffffffu, (uint32_t)__ldg(a.near_list + (int64_t)par * a.total_items + w), 0);
-        else if (a.mode == STREAM_FAR || FLIPS) mk = __ldg(mark + w);
+        } else if (far) {
+            // The force launch beside a FAR pass rewrites slots of near items
+            // (the link exchange), so nothing of a near item may be read here.
+            // Its mark is taken an item ahead, which keeps that load's latency
+            // off all items but a warp's first.
+            mk = mk_next;
+            if (w + nwarps < count) mk_next = __ldg(mark + w + nwarps);
+            if (__shfl_sync(0xffffffffu, mk, 0) == (int32_t)step64) continue;
+        } else if (FLIPS) {
+            mk = __ldg(mark + w);
+        }
         const int d = one ? 0 : (int)__ldg(a.item_dom + g);
         const DomDev& D = a.doms[d];
         const Geo G = one ? param_geo(a.dom0) : load_geo(D);
@@ -86,19 +98,19 @@ __global__ void __launch_bounds__(REG_K1_MAX_BLOCK, (k1_min_blocks<S, NOISE, PL>
                                reinterpret_cast<const char*>(base + yp * pitch)};
         // x-1 / x+V across a seam: wrapped when periodic; at open ends any
         // in-range element stands in until the Zou-He or corner patch.  Lanes
-        // beyond the row read chunk 0 and store nothing.
-        const int x0 = (seg * 32 + lane) * V;
+        // beyond the row read the segment's first chunk and store nothing.
+        const int x0 = (seg * 32 + lane) * V, xs = seg * 32 * V;
         const bool in_row = x0 < nx;
         int xl = x0 - 1, xr = x0 + V;
         if (xl < 0) xl = (G.flags & FLAG_PX) ? nx - 1 : 0;
         if (xr >= nx) xr = (G.flags & FLAG_PX) ? 0 : nx - 1;
-        const uint32_t xo = in_row ? (uint32_t)x0 * EB : 0u, xlo = in_row ? (uint32_t)xl * EB : 0u,
-                       xro = in_row ? (uint32_t)xr * EB : 0u;
+        const uint32_t xo = (uint32_t)(in_row ? x0 : xs) * EB, xlo = (uint32_t)(in_row ? xl : xs) * EB,
+                       xro = (uint32_t)(in_row ? xr : xs) * EB;
         // The flag words are loaded for every chunk, with the populations: a load
         // that waits for a bit of the row's mask first costs more than the 2 bytes
         // a node.
         uint16_t fl[V];
-        load_flags<V>(a.nflags + G.node_off + y * pitch + (in_row ? x0 : 0), fl);
+        load_flags<V>(a.nflags + G.node_off + y * pitch + (in_row ? x0 : xs), fl);
         Chunk<S> v[9];
         T e[9];
 #pragma unroll
@@ -111,8 +123,8 @@ __global__ void __launch_bounds__(REG_K1_MAX_BLOCK, (k1_min_blocks<S, NOISE, PL>
         const ExtPrm<A> X = load_ext<A, NOISE, PL>(one ? a.dom0 : D);
         W th[NP][6];
         chunk_thetas<S, NOISE, PL>(X, (uint32_t)(y * nx + x0), step, th);
-        const bool near_item = __shfl_sync(0xffffffffu, mk, 0) == (int32_t)step64;
-        if ((a.mode != STREAM_FAR || !near_item) && in_row) {
+        const bool near_item = FLIPS && __shfl_sync(0xffffffffu, mk, 0) == (int32_t)step64;
+        if (in_row) {
             W f[9][NP];
             form_chunk<S>(v, e, f, nx - 1 - x0);
             uint32_t any = 0;

@@ -1,0 +1,48 @@
+"""The overlapped chains of a step graph against the same launches one after another.
+
+A lattice of more work items than the split rule's runs its FAR passes beside the force
+launches, whose link exchange rewrites slots of the items near the disks.  Disks lie a few
+nodes from item borders and from the periodic seam, so that the FAR items beside them read up
+to the last node that the exchange leaves alone.  lbm_profile_steps runs every launch of a
+step after the one before it; populations and particle states must be the same bits.
+"""
+import numpy as np
+import pytest
+
+from gpu_helpers import gpu_params
+from paper_2006_12910_gb300 import lbm, workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True, scope="module")
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+
+
+@pytest.mark.parametrize("launch", [(1, 128, 0), (3, 128, 0), (2, 64, 2)])
+@pytest.mark.parametrize("store,kT", [("f64", 0.0), ("f32s", 0.0), ("f32s", 1e-6), ("f16s", 0.0)])
+def test_chains_equal_the_launches_in_sequence(store, kT, launch):
+    nx, ny, R = 516, 1000, 6.0
+    # left rims 0.3 to 9.3 nodes right of an item border (x = 128, 256), right rims left of one
+    # (x = 384) and of the seam; every one moves
+    parts = [dict(x=b + s * (R + 1.3 + k), y=60.0 + 90.0 * k + 25.0 * (j % 2), R=R, rho_p=1.1, U=0.02 * s, V=0.01)
+             for j, (b, s) in enumerate([(128, 1), (256, 1), (384, -1), (516, -1)]) for k in range(10)]
+    base = dict(nx=nx, ny=ny, periodic_x=1, periodic_y=0, walls_y=1, tau=0.8, gx=1e-6, lj_psi=1e-4, lj_rit=2.5,
+                kT=kT, seed=11)
+    f0 = workloads.random_populations(nx, ny, seed=3, amp=0.01)
+    got = []
+    for run in ("step", "profile_steps"):
+        ctx = lbm.Context(gpu_params(base, store, len(parts)), particles=[parts])
+        ctx.set_populations(f0)
+        ctx.set_launch(*launch)
+        for n in (1, 20, 7):
+            getattr(ctx, run)(n)
+        ctx.sync()
+        got.append((ctx.populations(), ctx.particles_array()))
+        ctx.close()
+    assert np.array_equal(got[0][0], got[1][0])
+    assert np.array_equal(got[0][1], got[1][1])
