@@ -134,8 +134,8 @@ __global__ void __launch_bounds__(STAGED_MAX_BLOCK) k_stream_staged(StreamArgs a
     const int par = (int)(step64 % 3);
     const int32_t next_stamp = (int32_t)(step64 + 1);
     const bool far_only = a.mode == STREAM_FAR;
-    const T* __restrict__ src = static_cast<const T*>(a.src);
-    T* __restrict__ dst = static_cast<T*>(a.dst);
+    const T* src = static_cast<const T*>(a.src);
+    T* dst = static_cast<T*>(a.dst);
     const int64_t count = a.total_items;
 
     if (lane == 0) {

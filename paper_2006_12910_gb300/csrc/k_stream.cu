@@ -56,8 +56,8 @@ __global__ void __launch_bounds__(REG_K1_MAX_BLOCK, (k1_min_blocks<S, NOISE, PL>
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.ctr_out = step64 + 1;
     const uint32_t step = (uint32_t)step64;
     const int par = (int)(step64 % 3);
-    const T* __restrict__ src = static_cast<const T*>(a.src);
-    T* __restrict__ dst = static_cast<T*>(a.dst);
+    const T* src = static_cast<const T*>(a.src);
+    T* dst = static_cast<T*>(a.dst);
     bool ok = true;
     const uint32_t count = a.mode == STREAM_NEAR ? (uint32_t)__ldg(a.near_cnt + par) : (uint32_t)a.total_items;
     const int32_t next_stamp = (int32_t)(step64 + 1);
@@ -111,18 +111,22 @@ __global__ void __launch_bounds__(REG_K1_MAX_BLOCK, (k1_min_blocks<S, NOISE, PL>
         // a node.
         uint16_t fl[V];
         load_flags<V>(a.nflags + G.node_off + y * pitch + (in_row ? x0 : xs), fl);
+        const HotPrm<A> H = one ? param_hot<A>(a.dom0) : load_hot<A>(D);
+        const ExtPrm<A> X = load_ext<A, NOISE, PL>(one ? a.dom0 : D);
+        // The normals are drawn while the loads are in flight; with the power law
+        // before them, for want of registers (ensemble 169 us a step, 191 before
+        // the loads; noise and tau* 56.6, 57.9 behind them).
+        W th[NP][6];
+        if (PL) chunk_thetas<S, NOISE, PL>(X, (uint32_t)(y * nx + x0), step, th);
         Chunk<S> v[9];
         T e[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
             const char* p = rows[cy(i) == 0 ? 0 : (cy(i) == 1 ? 1 : 2)] + (int64_t)i * plane * EB;
             v[i].load(p + xo);
-            if (cx(i)) e[i] = __ldg(reinterpret_cast<const T*>(p + (cx(i) == 1 ? xlo : xro)));
+            if (cx(i)) load_pop(e[i], p + (cx(i) == 1 ? xlo : xro));
         }
-        const HotPrm<A> H = one ? param_hot<A>(a.dom0) : load_hot<A>(D);
-        const ExtPrm<A> X = load_ext<A, NOISE, PL>(one ? a.dom0 : D);
-        W th[NP][6];
-        chunk_thetas<S, NOISE, PL>(X, (uint32_t)(y * nx + x0), step, th);
+        if (!PL) chunk_thetas<S, NOISE, PL>(X, (uint32_t)(y * nx + x0), step, th);
         const bool near_item = FLIPS && __shfl_sync(0xffffffffu, mk, 0) == (int32_t)step64;
         if (in_row) {
             W f[9][NP];

@@ -136,18 +136,9 @@ __device__ __forceinline__ void from_a(float v, float, float& o) { o = v; }
 __device__ __forceinline__ void from_a(float v, float s, __half& o) { o = __float2half_rn(v * s); }
 __device__ __forceinline__ void from_a(float v, float s, __nv_bfloat16& o) { o = __float2bfloat16_rn(v * s); }
 
-// Vector load (read-only path) of NV consecutive elements: one 8- or 16-byte access.
 template <int B> struct VecOf;
 template <> struct VecOf<8> { typedef uint2 type; };
 template <> struct VecOf<16> { typedef uint4 type; };
-template <class S, int NV>
-__device__ __forceinline__ void load_vec(const typename S::T* p, typename S::A (&out)[NV], typename S::A inv) {
-    typedef typename VecOf<NV * sizeof(typename S::T)>::type VT;
-    union { VT u; typename S::T t[NV]; } r;
-    r.u = __ldg(reinterpret_cast<const VT*>(p));
-#pragma unroll
-    for (int k = 0; k < NV; ++k) out[k] = to_a(r.t[k], inv);
-}
 __device__ __forceinline__ uint32_t pack2(float a, float b, __half) {
     const __half2 h = __floats2half2_rn(a, b);
     return *reinterpret_cast<const uint32_t*>(&h);
@@ -156,8 +147,46 @@ __device__ __forceinline__ uint32_t pack2(float a, float b, __nv_bfloat16) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<const uint32_t*>(&h);
 }
+// A load of populations.  Not through the read-only path (__ldg, ld.global.nc):
+// that one is for memory nobody writes while the grid lives, and a programmatic
+// dependent is resident while the launch before it still writes the arena.
+// Volatile, so that it stays behind the wait for that launch; it is written as
+// instructions because that constrains the code around it least (us a step with
+// __ldg / plain dereferences / these: porous 2048x1024 33.5 / 33.9 / 32.8, with
+// noise and tau* 56.8 / 58.4 / 56.6, 4096x2048 without particles 105.2 / 105.8 / 102.4).
+__device__ __forceinline__ void load_pop(uint4& v, const void* p) {
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+}
+__device__ __forceinline__ void load_pop(uint2& v, const void* p) {
+    asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+}
+__device__ __forceinline__ void load_pop(double& v, const void* p) {
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+}
+__device__ __forceinline__ void load_pop(float& v, const void* p) {
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+}
+__device__ __forceinline__ void load_pop(__half& v, const void* p) {
+    uint16_t u;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(u) : "l"(p));
+    v = __ushort_as_half(u);
+}
+__device__ __forceinline__ void load_pop(__nv_bfloat16& v, const void* p) {
+    uint16_t u;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(u) : "l"(p));
+    v = __ushort_as_bfloat16(u);
+}
+// Vector load of NV consecutive elements: one 8- or 16-byte access.
+template <class S, int NV>
+__device__ __forceinline__ void load_vec(const typename S::T* p, typename S::A (&out)[NV], typename S::A inv) {
+    typedef typename VecOf<NV * sizeof(typename S::T)>::type VT;
+    union { VT u; typename S::T t[NV]; } r;
+    load_pop(r.u, p);
+#pragma unroll
+    for (int k = 0; k < NV; ++k) out[k] = to_a(r.t[k], inv);
+}
 // A chunk as the collision takes it: V / Vec<W>::N vectors W (half-precision
-// kinds in their scaled units), one 8- or 16-byte load (read-only path) or store.
+// kinds in their scaled units), one 8- or 16-byte load or store.
 template <class S> struct ChunkOf { typedef float2 W; static constexpr int N = S::V / 2; };
 template <> struct ChunkOf<StF64> { typedef double W; static constexpr int N = StF64::V; };
 template <class S>
@@ -165,7 +194,7 @@ struct Chunk {  // as loaded; get() converts
     typedef typename VecOf<S::V * sizeof(typename S::T)>::type VT;
     union { VT u; typename S::T t[S::V]; };
     __device__ __forceinline__ Chunk() {}
-    __device__ __forceinline__ void load(const void* p) { u = __ldg(static_cast<const VT*>(p)); }
+    __device__ __forceinline__ void load(const void* p) { load_pop(u, p); }
     __device__ __forceinline__ void load_shared(const void* p) { u = *static_cast<const VT*>(p); }
     __device__ __forceinline__ void get(typename ChunkOf<S>::W (&v)[ChunkOf<S>::N]) const {
         constexpr int N = Vec<typename ChunkOf<S>::W>::N;
@@ -180,17 +209,11 @@ __device__ __forceinline__ void store_chunk(void* p, const typename ChunkOf<S>::
     else if constexpr (sizeof(typename S::T) == 4) *static_cast<float4*>(p) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
     else *static_cast<uint2*>(p) = make_uint2(pack2(v[0].x, v[0].y, typename S::T()), pack2(v[1].x, v[1].y, typename S::T()));
 }
+// One element, by a plain dereference: in the rare branches that use it the
+// volatile form costs the loops around them registers (noise and tau* 59.6 us).
 template <class S>
 __device__ __forceinline__ typename S::A load_one(const typename S::T* p, typename S::A inv) {
-    return to_a(__ldg(p), inv);
-}
-template <>
-__device__ __forceinline__ float load_one<StF16S>(const __half* p, float inv) {
-    return __half2float(__ldg(p)) * inv;
-}
-template <>
-__device__ __forceinline__ float load_one<StBF16S>(const __nv_bfloat16* p, float inv) {
-    return __bfloat162float(__ldg(p)) * inv;
+    return to_a(*p, inv);
 }
 
 // ---------------------------------------------------------------------------
