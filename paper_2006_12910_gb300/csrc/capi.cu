@@ -421,6 +421,7 @@ PartArgs part_args(lbm_ctx* c, int cur) {
     a.diag = c->diag;
     a.err = c->err;
     a.ctr = c->ctr + cur;
+    a.par = (int)(c->steps ^ c->cur ^ cur) & 1;  // every step turns over the arena and the step count
     a.pstep = c->pstep + cur;
     a.mark = c->mark;
     a.near_list = c->near_list;
@@ -1399,6 +1400,7 @@ int lbm_load(lbm_ctx* c, const char* path) {
         c->flips_total = h.flips_total;
         for (int d = 0; d < c->ndom; ++d) c->hd[d].np = dnp[d];
         c->np_active = np_total;
+        c->steps = h.steps;  // the set-up launches take the step's parity from it
         CKC(c, cudaMemcpy(c->dd, c->hd.data(), sizeof(DomDev) * c->ndom, cudaMemcpyHostToDevice));
         CKC(c, cudaMemset(c->mark, 0xff, sizeof(int32_t) * 3 * std::max<int64_t>(1, c->total_items)));
         CKC(c, cudaMemset(c->near_cnt, 0, sizeof(int32_t) * 3));

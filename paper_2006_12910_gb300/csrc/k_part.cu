@@ -423,20 +423,22 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(c
     const int rel = (int)blockIdx.x / a.np;
     const int role = role0 + rel;
     const int p = (int)blockIdx.x - rel * a.np;
-    // Independent loads first (step counter, static data, both parities of
-    // the state), so the prologue waits for one round trip, then the domain.
+    // Independent loads first (step counter, static data, state), so the prologue
+    // waits for one round trip, then the domain.
     // PL_AHEAD: launched after role A of step t-1 for step t (or t+1), whose
-    // state counter is not yet published: t from the word role A stored.
+    // state counter is not yet published: t from the word role A stored.  The
+    // copies of the other parity belong to launches that may run beside this
+    // one (role A of the next step writes the state, the rasterisation of the
+    // step before the list lengths) and are not touched.
     const int64_t t = (modes & PL_AHEAD) ? *a.pstep : *a.ctr;
+    const int par = (modes & PL_AHEAD) ? a.par ^ 1 : a.par;  // t & 1
     const PartStatic st = a.st[p];
-    const PartState q0 = a.state[p], q1 = a.state[(int64_t)a.np + p];
-    // role A: the list lengths of both parities in the same round trip
-    int nl2[2] = {0, 0}, nf2[2] = {0, 0};
+    const PartState q = a.state[(int64_t)par * a.np + p];
+    // role A: the list lengths in the same round trip
+    int nl = 0, nf = 0;
     if (LO == 0 && role == 0) {
-        nl2[0] = a.nlinks[p];
-        nl2[1] = a.nlinks[(int64_t)a.np + p];
-        nf2[0] = a.nflips[p];
-        nf2[1] = a.nflips[(int64_t)a.np + p];
+        nl = a.nlinks[(int64_t)par * a.np + p];
+        nf = a.nflips[(int64_t)par * a.np + p];
     }
     const bool advance = modes & PL_ADVANCE;
     // The near-item list of step t+2 is touched by nobody during this step.
@@ -452,9 +454,7 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(c
     // a copy would put all of it (0.6 KB) into every thread's local memory.
     typename std::conditional<HI == 0, const DomDev, const DomDev&>::type D = a.one_domain ? a.dom0 : a.doms[st.dom];
     if (p - D.p0 >= D.np) return;
-    const int par = (int)(t & 1);
     const PartState* S0 = a.state + (int64_t)par * a.np;
-    const PartState q = par ? q1 : q0;
     const double R = st.R;
     const bool px = D.flags & FLAG_PX, py = D.flags & FLAG_PY;
     typename S::T* base = static_cast<typename S::T*>(a.arena) + D.off;
@@ -511,7 +511,6 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(c
         __shared__ double newst[6], xmid[3], zval[6];
         const int32_t* links = a.links + (int64_t)par * a.links_total;
         const int32_t* flips = a.flips + (int64_t)par * a.flips_total;
-        const int nl = nl2[par], nf = nf2[par];
         const bool forces = modes & PL_FORCES, swap = modes & PL_SWAP;
         // one round of four links per thread covers nl <= 512: the decoded links
         // and slot values then stay in registers from phase 1 to phase 3

@@ -113,6 +113,7 @@ struct PartArgs {
     double* diag;              // np * DIAG_N
     unsigned* err;
     const int64_t* ctr;        // step counter of the state in `arena`
+    int par;                   // its parity, which the host knows: the copies to read, before the counter arrives
     // The force launch of step t from `arena` stores t + 1 here; the launches
     // for later steps that follow it read it instead of a state counter that
     // a concurrent stream-collide pass may already have advanced.  One word

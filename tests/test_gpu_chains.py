@@ -46,3 +46,30 @@ def test_chains_equal_the_launches_in_sequence(store, kT, launch):
         ctx.close()
     assert np.array_equal(got[0][0], got[1][0])
     assert np.array_equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("before", [0, 1, 2])
+def test_restored_at_an_odd_step(before, tmp_path):
+    """The launches take the step's parity (their copies of states and lists) from the host;
+    a checkpoint of step 7 restored into a context that has itself done 0, 1 or 2 steps
+    continues as the run it was taken from."""
+    base = dict(nx=96, ny=64, periodic_x=1, periodic_y=1, walls_y=0, tau=0.8, gx=1e-5, lj_psi=1e-4, lj_rit=2.5)
+    parts = [dict(x=30.2, y=30.7, R=7.3, rho_p=1.2, U=0.05, V=-0.03, Omega=0.003),
+             dict(x=60.6, y=33.1, R=6.1, rho_p=0.9, U=-0.04, V=0.02)]
+
+    def ctx():
+        c = lbm.Context(gpu_params(base, "f32s", 2), particles=[parts])
+        c.set_populations(workloads.random_populations(96, 64, seed=9, amp=0.01))
+        return c
+
+    a, b = ctx(), ctx()
+    a.step(7)
+    a.save(tmp_path / "ck.bin")
+    b.step(before)
+    b.load_checkpoint(tmp_path / "ck.bin")
+    for n in (1, 4, 6):
+        a.step(n)
+        b.step(n)
+    assert b.step_count == 18
+    assert np.array_equal(a.populations(), b.populations())
+    assert a.particles() == b.particles()
