@@ -1002,6 +1002,7 @@ int lbm_add_particles(lbm_ctx* c, int dom, int n, const lbm_particle* p) {
     CKC(c, dev_malloc(&c->diag, sizeof(double) * DIAG_N * ns));
     CKC(c, dev_malloc(&c->ljf, sizeof(double) * 2 * 4 * ns));
     CKC(c, cudaMemset(c->ljf, 0, sizeof(double) * 2 * 4 * ns));
+    CKC(c, cudaMemset(c->flipmom, 0, sizeof(double) * 2 * 3 * std::max<int64_t>(fo, 1)));
     CKC(c, cudaMemset(c->nlinks, 0, sizeof(int32_t) * 2 * ns));
     CKC(c, cudaMemset(c->nflips, 0, sizeof(int32_t) * 2 * ns));
     CKC(c, cudaMemset(c->diag, 0, sizeof(double) * DIAG_N * ns));
@@ -1378,6 +1379,7 @@ int lbm_load(lbm_ctx* c, const char* path) {
         c->hstate = s;
         CKC(c, dev_malloc(&c->pstate, sizeof(PartState) * 2 * ns));
         CKC(c, dev_malloc(&c->flipmom, 2 * 8 * fm.size()));
+        CKC(c, cudaMemset(c->flipmom, 0, 2 * 8 * fm.size()));
         CKC(c, dev_malloc(&c->pst, sizeof(PartStatic) * ns));
         CKC(c, dev_malloc(&c->links, 2 * 4 * L.size()));
         CKC(c, dev_malloc(&c->flips, 2 * 4 * F.size()));

@@ -115,6 +115,16 @@ __device__ __forceinline__ Box disk_box(const DiskF& k) {
     b.h = k.cy + (int)ceilf(k.fy + r) + 1 - b.y0 + 1;
     return b;
 }
+// The box b of a disk at t+1 in the image nearest to o, its box at t: the centre
+// is stored wrapped, so when it crosses a periodic seam the two boxes lie at
+// opposite ends of the domain, and a union over the period would hold both
+// images of every node.  (A disk moves by less than a node a step and its box is
+// narrower than the period.)
+__device__ __forceinline__ Box box_beside(const DomDev& D, Box b, const Box& o) {
+    if (D.flags & FLAG_PX) b.x0 += 2 * (b.x0 - o.x0) > D.nx ? -D.nx : (2 * (o.x0 - b.x0) > D.nx ? D.nx : 0);
+    if (D.flags & FLAG_PY) b.y0 += 2 * (b.y0 - o.y0) > D.ny ? -D.ny : (2 * (o.y0 - b.y0) > D.ny ? D.ny : 0);
+    return b;
+}
 // Integer minimum image, in [-L/2, L/2), of a node offset along a periodic
 // axis.  Offsets here (a node within R + 8 of the domain against a centre in
 // it, with 2R + 8 below the period) are under 5L/2 in magnitude, so two
@@ -1170,7 +1180,7 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(c
         constexpr int mx = 16 / (int)sizeof(typename S::T);
         const int mpar = (int)(t_next % 3);  // three-way: the passes of t and t+1 read the other two
         const int lpar = (int)(t_next % 3);
-        const Box bo = uni.bo, bn = uni.bn;
+        const Box bo = uni.bo, bn = box_beside(D, uni.bn, bo);
         int x0 = min(bo.x0, bn.x0) - mx, x1 = max(bo.x0 + bo.w, bn.x0 + bn.w) + mx - 1;
         if (px && x1 - x0 >= D.nx) {  // once around: every item of the rows
             x0 = 0;
@@ -1256,7 +1266,7 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(c
     }
     // Union of the old and new boxes; every neighbour of a node inside either
     // disk lies in it.
-    const Box bo = uni.bo, bn = uni.bn;
+    const Box bo = uni.bo, bn = box_beside(D, uni.bn, bo);
     Box U;
     U.x0 = min(bo.x0, bn.x0);
     U.y0 = min(bo.y0, bn.y0);
