@@ -114,7 +114,8 @@ int lbm_create_ensemble(int ndom, const lbm_params* per_domain, void* cuda_strea
 /* Stationary solid nodes of domain dom (Sec. 3 "inline obstacles"):
  * solid[y*nx + x] != 0 marks a solid node.  Copied.  Solid nodes hold no
  * populations; their neighbours bounce back halfway.  Must precede
- * lbm_add_particles. */
+ * lbm_add_particles.  On a context that holds a state, nodes that stay fluid
+ * keep theirs and nodes that turn fluid start at rest with density rho0. */
 int lbm_set_geometry(lbm_ctx* ctx, int dom, const uint8_t* solid);
 
 /* Add n particles to domain dom (copied) and rasterise them (Sec. 3, Fig. 1:

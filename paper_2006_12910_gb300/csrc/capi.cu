@@ -662,12 +662,20 @@ int ensure_stage(lbm_ctx* c, size_t bytes) {
     return LBM_OK;
 }
 
-// Solid bytes, flag words and chunk bits of one domain from its host mask.
-int upload_geometry(lbm_ctx* c, int dom) {
+// Solid bytes of one domain as the kernels read them, from its host mask.
+std::vector<uint8_t> pitched_solid(const lbm_ctx* c, int dom) {
     const DomDev& D = c->hd[dom];
     const std::vector<uint8_t>& hs = c->hsolid[dom];
     std::vector<uint8_t> pitched((size_t)D.plane, 0);
     for (int y = 0; y < D.ny; ++y) memcpy(&pitched[(size_t)y * D.pitch], &hs[(size_t)y * D.nx], D.nx);
+    return pitched;
+}
+
+// Solid bytes, flag words and chunk bits of one domain from its host mask.
+int upload_geometry(lbm_ctx* c, int dom) {
+    const DomDev& D = c->hd[dom];
+    const std::vector<uint8_t>& hs = c->hsolid[dom];
+    const std::vector<uint8_t> pitched = pitched_solid(c, dom);
     std::vector<uint16_t> fl;
     std::vector<uint32_t> words;
     build_flags(D, hs.data(), fl, words);
@@ -924,16 +932,20 @@ int lbm_set_geometry(lbm_ctx* c, int dom, const uint8_t* solid) {
     if (!solid) return fail(c, LBM_E_INVAL, "solid mask is NULL");
     if (c->np_active > 0) return fail(c, LBM_E_STATE, "set the geometry before adding particles");
     const DomDev& D = c->hd[dom];
+    r = ensure_stage(c, (size_t)D.plane);
+    if (r) return r;
     std::vector<uint8_t>& hs = c->hsolid[dom];
     for (size_t k = 0; k < hs.size(); ++k) hs[k] = solid[k] ? 1 : 0;
     CKC(c, cudaStreamSynchronize(c->stream));
+    // The slots of solid nodes hold what the passes stored there and mean
+    // nothing: the state is re-applied from the old mask and the new one.
+    const std::vector<uint8_t> now = pitched_solid(c, dom);
+    uint8_t* d_now = reinterpret_cast<uint8_t*>(c->d_stage);
+    CKC(c, cudaMemcpy(d_now, now.data(), now.size(), cudaMemcpyHostToDevice));
+    CKC(c, launch_resolid(c->kind, D, c->f[c->cur], c->solid + D.node_off, d_now, c->stream));
+    CKC(c, cudaStreamSynchronize(c->stream));
     r = upload_geometry(c, dom);
     if (r) return r;
-    // solid nodes hold no populations: re-apply the current state with zeros there
-    r = ensure_stage(c, sizeof(double) * 9 * (size_t)D.nx * D.ny);
-    if (r) return r;
-    CKC(c, launch_export(c->kind, D, c->f[c->cur], c->solid, c->d_stage, c->stream));
-    CKC(c, launch_import(c->kind, D, c->d_stage, c->f[c->cur], c->solid, c->stream));
     return sync_and_check(c);
 }
 

@@ -36,6 +36,20 @@ __global__ void k_fill_rest(DomDev D, typename S::T* arena, const uint8_t* solid
     }
 }
 
+template <class S>
+__global__ void k_resolid(DomDev D, typename S::T* arena, const uint8_t* was, const uint8_t* now) {
+    const int64_t n = (int64_t)D.ny * D.pitch;
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
+        if (k % D.pitch >= D.nx || !(was[k] | now[k])) continue;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            typename S::T* p = arena + D.off + (int64_t)i * D.plane + k;
+            if (now[k]) from_a((typename S::A)0, (typename S::A)1, *p);
+            else store_full<S>(p, D, i, wgt(i) * D.rho0);
+        }
+    }
+}
+
 __global__ void k_lj_wall(DomDev D, const uint8_t* solid, const LjEntry* tab, const int32_t* cnt, int dom, double2* out) {
     const int64_t n = (int64_t)D.nx * D.ny;
     const int m = cnt[dom];
@@ -366,6 +380,13 @@ cudaError_t launch_fill_rest(int kind, const DomDev*, int ndom, const DomDev* hd
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
+}
+
+cudaError_t launch_resolid(int kind, const DomDev& D, void* arena, const uint8_t* was, const uint8_t* now,
+                           cudaStream_t s) {
+    const int64_t nb = blocks_for((int64_t)D.ny * D.pitch, 256);
+    LBM_DISPATCH(kind, (k_resolid<S><<<(unsigned)nb, 256, 0, s>>>(D, static_cast<S::T*>(arena), was, now)));
+    return cudaGetLastError();
 }
 
 cudaError_t launch_lj_wall(const DomDev& D, const uint8_t* solid, const LjEntry* tab, const int32_t* cnt, int dom,

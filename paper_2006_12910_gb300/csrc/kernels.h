@@ -73,6 +73,9 @@ cudaError_t launch_fill_rest(int kind, const DomDev* doms, int ndom, const DomDe
 // offsets wrap on periodic axes; beyond an open end there is no wall).
 cudaError_t launch_lj_wall(const DomDev& D, const uint8_t* solid, const LjEntry* tab, const int32_t* cnt, int dom,
                            double2* out, cudaStream_t s);
+// Stored populations of one domain when its solid bytes (a node each, at y * pitch + x)
+// change from was to now: zeros in solid nodes, rest in nodes that turn fluid.
+cudaError_t launch_resolid(int kind, const DomDev& D, void* arena, const uint8_t* was, const uint8_t* now, cudaStream_t s);
 // Host-order FP64 f[9][ny][nx] (device buffer) -> stored populations of one domain.
 cudaError_t launch_import(int kind, const DomDev& D, const double* in, void* arena, const uint8_t* solid,
                           cudaStream_t s);
