@@ -208,7 +208,9 @@ int validate(const lbm_params& p, int d, lbm_ctx* c) {
 
 int64_t round_up(int64_t a, int64_t b) { return (a + b - 1) / b * b; }
 
-void fill_dom(DomDev& D, const lbm_params& p, int kind) {
+// pl: the kernels of the context are the power-law variants (some domain of it
+// has the power law).
+void fill_dom(DomDev& D, const lbm_params& p, int kind, bool pl) {
     memset(&D, 0, sizeof D);
     D.nx = p.nx;
     D.ny = p.ny;
@@ -267,7 +269,7 @@ void fill_dom(DomDev& D, const lbm_params& p, int kind) {
     D.drho_in_f = (float)D.drho_in; D.drho_out_f = (float)D.drho_out; D.kT_f = (float)D.kT;
     D.n_pl_f = (float)D.n_pl; D.xi_pl_f = (float)D.xi_pl; D.tau_min_f = (float)D.tau_min;
     D.tau_max_f = (float)D.tau_max; D.tmin_pow_f = (float)D.tmin_pow; D.tmax_pow_f = (float)D.tmax_pow;
-    D.var = 3.0 * D.kT * (p.power_law ? 1.0 : D.inv_tau * (2.0 - D.inv_tau));
+    D.var = 3.0 * D.kT * (pl ? 1.0 : D.inv_tau * (2.0 - D.inv_tau));
     D.var_f = (float)D.var; D.var_lo_f = (float)(D.var - (double)D.var_f);
     D.scale_f = (float)D.scale; D.inv_scale_f = (float)D.inv_scale;
     {
@@ -735,9 +737,10 @@ int lbm_create_ensemble(int ndom, const lbm_params* per_domain, void* cuda_strea
     std::vector<uint16_t> item_dom;
     int64_t off = 0, node_off = 0, mask_off = 0, items = 0;
     int pslot = 0;
+    for (int d = 0; d < ndom; ++d) c->pl |= per_domain[d].power_law != 0;
     for (int d = 0; d < ndom; ++d) {
         DomDev& D = c->hd[d];
-        fill_dom(D, per_domain[d], c->kind);
+        fill_dom(D, per_domain[d], c->kind, c->pl);
         D.off = off + (per_domain[d].walls_y ? D.pitch : 0);  // row 0 of plane 0, after the ghost row
         D.node_off = node_off;
         D.mask_off = mask_off;
@@ -752,7 +755,6 @@ int lbm_create_ensemble(int ndom, const lbm_params* per_domain, void* cuda_strea
         pslot += per_domain[d].max_particles;
         c->hsolid[d].assign((size_t)D.nx * D.ny, 0);
         c->noise |= per_domain[d].kT > 0.0;
-        c->pl |= per_domain[d].power_law != 0;
     }
     c->arena_elems = (size_t)off;
     c->node_bytes = (size_t)node_off;

@@ -71,8 +71,8 @@ struct alignas(16) DomDev {
     // FP32 copies of the collision parameters, so the FP32 path converts nothing
     float tau_f, inv_tau_f, rho0_f, gx_f, gy_f, rho_in_f, rho_out_f, drho_in_f, drho_out_f, kT_f;
     float n_pl_f, xi_pl_f, tau_min_f, tau_max_f, tmin_pow_f, tmax_pow_f, scale_f, inv_scale_f;
-    // noise variance of Eq. NP2 over rho: 3 kT omega (2 - omega), with the power
-    // law 3 kT; FP32 as a pair hi + lo
+    // noise variance of Eq. NP2 over rho: 3 kT omega (2 - omega), or 3 kT where the
+    // context's kernels are the power-law variants; FP32 as a pair hi + lo
     float var_f, var_lo_f;
 };
 
