@@ -255,6 +255,10 @@ void fill_dom(DomDev& D, const lbm_params& p, int kind, bool pl) {
     D.tau_min = p.tau_min;
     D.tau_max = p.tau_max;
     D.n_is_one = p.power_law ? (p.n_pl == 1.0) : 1;
+    if (pl && !p.power_law) {  // a Newtonian domain among power-law ones: tau* is its tau
+        D.xi_pl = (p.tau - 0.5) / 3.0;
+        D.tau_min = D.tau_max = p.tau;
+    }
     if (p.power_law) {
         D.tmin_pow = std::pow(p.tau_min, 1.0 - p.n_pl);
         D.tmax_pow = std::pow(p.tau_max, 1.0 - p.n_pl);

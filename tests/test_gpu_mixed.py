@@ -52,3 +52,11 @@ def test_noise_variance(store, first):
     """xi = (tau - 1/2) / 3 is the viscosity the kernels take tau from."""
     errs = run(store, lambda tau: dict(xi_pl=(tau - 0.5) / 3, tau_min=0.51, tau_max=2.0), first)
     assert max(errs) < LIMIT[store], errs
+
+
+@pytest.mark.parametrize("given", [dict(), dict(xi_pl=0.3, tau_min=0.51, tau_max=0.7, n_pl=0.5)])
+@pytest.mark.parametrize("store", list(LIMIT))
+def test_own_relaxation_time(store, given):
+    """Power-law parameters of a domain without the power law, the defaults or any others, do nothing."""
+    errs = run(store, lambda tau: given, 1)
+    assert max(errs) < LIMIT[store], errs
