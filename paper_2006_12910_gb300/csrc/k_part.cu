@@ -753,19 +753,7 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(c
                                  cil = fma(aij, ajl, -(ail * ajj));
                     const double det = fma(ail, cil, fma(aij, cij, aii * cii));
                     const double num = fma(cil, sys[6 + l], fma(cij, sys[6 + j], cii * sys[6 + i]));
-                    // 1 / det: the hardware approximation times 1 + e + e^2, and the
-                    // quotient corrected by its remainder (the division far from 1)
-                    double y;
-                    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(det));
-                    const int ex = (__double2hiint(det) >> 20) & 0x7ff;
-                    if (ex > 200 && ex < 1800) {
-                        const double e = fma(-det, y, 1.0);
-                        y = fma(y, fma(e, e, e), y);
-                        const double x0 = num * y;
-                        xm = fma(fma(-det, x0, num), y, x0);
-                    } else {
-                        xm = num * (1.0 / det);
-                    }
+                    xm = num / det;
                     vn = fma(2.0, xm, -vn);
                 }
                 // A particle faster than a node per step, or a state that is no
