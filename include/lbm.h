@@ -138,8 +138,9 @@ int lbm_get_populations(lbm_ctx* ctx, int dom, double* f);
 /* Advance every domain by nsteps timesteps (Eqs. e.LB1, MP1-MP8, NP1-NP2,
  * nn5 per step).  Enqueued on the context stream (replayed as CUDA graphs:
  * one graph of exactly nsteps steps when lbm_prepare_steps prepared that
- * count, else one graph per binary digit of nsteps, up to 64 steps each; a
- * graph is built when a call first needs it); returns without waiting. */
+ * count, else one graph per binary digit of nsteps, up to 64 steps each; all
+ * are built by the first call, or by lbm_prepare_steps, after a change of the
+ * context); returns without waiting. */
 int lbm_step(lbm_ctx* ctx, int64_t nsteps);
 
 /* Per-step particle trajectories without a host round trip per step (the

@@ -4,8 +4,8 @@
 // f*(t) and the next state), per-node solid bytes and flag words, the per-chunk
 // flag bits, the step counters, a sticky error word and the particle arrays.
 // lbm_step replays CUDA graphs of 2^j timesteps, j = 0 .. GRAPH_LOG (the
-// binary digits of the step count, largest first), each built when a call first
-// needs it, or one graph of a count that lbm_prepare_steps prepared; a timestep is
+// binary digits of the step count, largest first) or one graph of a count that
+// lbm_prepare_steps prepared; a timestep is
 //   [particle forces + Newton-Euler + link exchange]
 //   -> [fused pull-stream + collide over every domain], beside it
 //   [re-rasterise, Eq. MP2 sums for later steps]
@@ -603,23 +603,25 @@ int capture_steps(lbm_ctx* c, int k, int nsteps, cudaGraphExec_t* out) {
     return LBM_OK;
 }
 
-// Graphs are built when a call first needs them: instantiating the whole set
-// (2 x 127 steps) took most of a small context's set-up (128x128 with one disk
-// and one prepared count 8.0 ms in all, 2.1 so; 2048x1024 porous 51 and 43).
-void drop_graphs(lbm_ctx* c) {
-    auto drop = [](cudaGraphExec_t& g) {
-        if (g) cudaGraphExecDestroy(g);
-        g = nullptr;
-    };
+// All graphs at once, when the first step (or lbm_prepare_steps) after a change
+// needs one: a later step of any count only launches.  Building each when a
+// call first needed it made set-up with one prepared count 2 to 9 ms shorter
+// (128x128 with one disk 2.1 against 4.4 ms, 2048x1024 porous 40 against 50) and
+// put captures, and their failures, into running simulations.
+int build_graphs(lbm_ctx* c) {
     for (int k = 0; k < 2; ++k) {
-        for (auto& g : c->gexec[k]) drop(g);
-        for (auto& g : c->gprep[k]) drop(g);
+        for (int j = 0; j <= GRAPH_LOG; ++j) {
+            const int r = capture_steps(c, k, 1 << j, &c->gexec[k][j]);
+            if (r) return r;
+        }
         c->gprep[k].resize(c->prepared.size(), nullptr);
+        for (size_t i = 0; i < c->prepared.size(); ++i) {
+            const int r = capture_steps(c, k, (int)c->prepared[i], &c->gprep[k][i]);
+            if (r) return r;
+        }
     }
     c->graph_dirty = false;
-}
-int ensure_graph(lbm_ctx* c, int k, int nsteps, cudaGraphExec_t* g) {
-    return *g ? LBM_OK : capture_steps(c, k, nsteps, g);
+    return LBM_OK;
 }
 
 // Pinned host block: the error word in the first PIN_HEAD bytes, then
@@ -1084,24 +1086,19 @@ int lbm_step(lbm_ctx* c, int64_t nsteps) {
     if (!c) return LBM_E_INVAL;
     if (nsteps < 0) return fail(c, LBM_E_INVAL, "nsteps must be >= 0");
     if (nsteps == 0) return LBM_OK;
-    if (c->graph_dirty) drop_graphs(c);
-    int r = LBM_OK;
+    if (c->graph_dirty) {
+        int r = build_graphs(c);
+        if (r) return r;
+    }
     for (size_t i = 0; i < c->prepared.size(); ++i) {
-        if (c->prepared[i] != nsteps) continue;
-        if ((r = ensure_graph(c, c->cur, (int)nsteps, &c->gprep[c->cur][i]))) return r;
+        if (c->prepared[i] != nsteps || i >= c->gprep[c->cur].size() || !c->gprep[c->cur][i]) continue;
         CKC(c, cudaGraphLaunch(c->gprep[c->cur][i], c->stream));
         c->cur ^= (int)(nsteps & 1);
         c->steps += nsteps;
         c->pstate_evt = c->np_active > 0;
         return LBM_OK;
     }
-    // every graph of the call exists before the first is launched (a failed
-    // capture leaves the state as it was)
-    const int64_t full = nsteps >> GRAPH_LOG;
-    if (full > 0 && (r = ensure_graph(c, c->cur, 1 << GRAPH_LOG, &c->gexec[c->cur][GRAPH_LOG]))) return r;
-    for (int j = GRAPH_LOG - 1; j >= 0; --j)
-        if (((nsteps >> j) & 1) && (r = ensure_graph(c, c->cur, 1 << j, &c->gexec[c->cur][j]))) return r;
-    for (int64_t n = full; n > 0; --n)  // even step counts: the state stays in arena cur
+    for (int64_t n = nsteps >> GRAPH_LOG; n > 0; --n)  // even step counts: the state stays in arena cur
         CKC(c, cudaGraphLaunch(c->gexec[c->cur][GRAPH_LOG], c->stream));
     for (int j = GRAPH_LOG - 1; j >= 0; --j) {
         if (!((nsteps >> j) & 1)) continue;
@@ -1141,23 +1138,25 @@ int lbm_prepare_steps(lbm_ctx* c, int64_t nsteps) {
     if (!c) return LBM_E_INVAL;
     if (nsteps < 1 || nsteps > LBM_PREPARE_MAX_STEPS)
         return fail(c, LBM_E_INVAL, "nsteps must be in 1 .. LBM_PREPARE_MAX_STEPS");
-    if (c->graph_dirty) drop_graphs(c);
-    size_t i = 0;
-    while (i < c->prepared.size() && c->prepared[i] != nsteps) ++i;
-    if (i == c->prepared.size()) {
-        if ((int)c->prepared.size() >= LBM_PREPARE_SLOTS) {  // drop the oldest
-            for (auto& gk : c->gprep) {
-                if (gk[0]) cudaGraphExecDestroy(gk[0]);
-                gk.erase(gk.begin());
-            }
-            c->prepared.erase(c->prepared.begin());
-            --i;
-        }
-        c->prepared.push_back(nsteps);
-        for (auto& gk : c->gprep) gk.resize(c->prepared.size(), nullptr);
-    }
     int r = LBM_OK;
-    for (int k = 0; k < 2 && !r; ++k) r = ensure_graph(c, k, (int)nsteps, &c->gprep[k][i]);
+    for (int64_t n : c->prepared)
+        if (n == nsteps) return c->graph_dirty && (r = build_graphs(c)) ? r : sync_and_check(c);
+    if ((int)c->prepared.size() >= LBM_PREPARE_SLOTS) {  // drop the oldest
+        for (auto& gk : c->gprep) {
+            if (!gk.empty() && gk[0]) cudaGraphExecDestroy(gk[0]);
+            if (!gk.empty()) gk.erase(gk.begin());
+        }
+        c->prepared.erase(c->prepared.begin());
+    }
+    c->prepared.push_back(nsteps);
+    if (c->graph_dirty) {
+        r = build_graphs(c);
+    } else {
+        for (int k = 0; k < 2 && !r; ++k) {
+            c->gprep[k].resize(c->prepared.size(), nullptr);
+            r = capture_steps(c, k, (int)nsteps, &c->gprep[k].back());
+        }
+    }
     return r ? r : sync_and_check(c);
 }
 
