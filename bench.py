@@ -609,11 +609,12 @@ def main():
     elif not args.no_autotune:
         ctx.autotune(20)
     # with particles: FAR and NEAR stream-collide passes, the particle force launch, the
-    # rasterisation + marks launch and the Eq. MP2 launch; lattices of fewer than 3,072 work
-    # items (rows of 32 chunks: 32 nodes in FP64, 128 otherwise) take one pass, the force
-    # launch and one launch for the rest
+    # rasterisation + marks launch and, with an Eq. MP2 force, its launch; lattices of at most
+    # 3,072 work items (rows of 32 chunks: 32 nodes in FP64, 128 otherwise) take one pass, the
+    # force launch and one launch for the rest
     items = w.ny * -(-w.nx // (32 if args.store == "f64" else 128))
-    kernels_per_step = (5 if items >= 3072 else 3) if w.particles else 1
+    lj = w.params.get("lj_psi", 0.0) > 0.0 and w.params.get("lj_rit", 2.5) > 0.0
+    kernels_per_step = ((5 if lj else 4) if items > 3072 else 3) if w.particles else 1
 
     def barrier():
         if world > 1:

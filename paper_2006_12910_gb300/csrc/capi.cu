@@ -494,16 +494,29 @@ cudaError_t enqueue_step(lbm_ctx* c, int cur, cudaStream_t s, bool pdl) {
 // force launches overlap the bulk of the lattice, and the Eq. MP2 sums (where
 // any domain has them) run on a stream of their own: beside a FAR pass their
 // CTAs would hold back the rasterisation (merged: 831 us a call of 20 steps of
-// the porous workload, 760 apart).  Below, one pass over every item after the
-// force launch ends as early as the near items alone would, and two chains
-// instead of four leave room for other contexts: the device has eight hardware
-// queues by default, and three contexts with four chains each waited for one
-// another (512x512 fluctuating box, calls of 20 steps of three contexts in
-// turn: 201 -> 146 us a call, one context alone 379 -> 386; 3000x41 channel 188
-// -> 131 and 372 -> 368).  SPLIT_ITEMS lies where the whole pass stops being the
-// shorter one (us a step, one context alone, whole / split: 512x512 noise,
-// 2,048 items, 18.0 / 18.2; 820x510 grains, 3,570 items, 21.3 / 23.6; 768x768
-// noise, 4,608 items, 22.4 / 18.8; 1300x820 grains, 9,020 items, 31.8 / 27.5).
+// the porous workload, 760 apart, when this was chosen).  Up to SPLIT_ITEMS, one
+// pass over every item after the force launch ends nearly as early as the near
+// items alone would, and two chains instead of four leave room for other
+// contexts: the device has eight hardware queues by default, and three contexts
+// with four chains each wait for one another.  The line lies where the split
+// begins to pay both for one context alone and for three in turn: between 2,400
+// and 2,880 items in FP32, between 2,400 and 9,600 of the shorter FP64 ones, one
+// value for all kinds (us a step, alone | three, whole against split):
+//   FP32 (an item: 128 nodes)
+//     2,048 items, 512x512 noise, 1 disk      14.5 |  6.0   15.0 |  6.1
+//     2,400 items, 640x480 porous, 3 disks    15.6 |  6.1   15.2 |  8.1
+//     2,400 items, 700x400 grains, 35 disks   16.2 |  9.1   15.5 |  9.6
+//     2,880 items, 576x576 noise, 1 disk      15.9 |  7.5   14.8 |  6.6
+//     3,570 items, 820x510 grains, 45 disks   17.3 | 11.5   15.9 | 10.6
+//     4,480 items, 900x560 porous, 5 disks    17.3 | 10.3   15.5 |  9.6
+//     8,192 items, 1024x1024 noise, 1 disk    26.2 | 18.3   18.8 | 16.5
+//   FP16 (128 nodes), porous
+//     2,400 items, 3 disks                    14.8 |  5.5   14.8 |  7.5
+//     5,600 items, 7 disks                    17.5 |  8.7   15.3 |  8.7
+//   FP64 (32 nodes), porous
+//     2,400 items, 1 disk                     12.1 |  5.0   12.4 |  6.9
+//     4,620 items, 1 disk                     16.2 |  7.6   15.4 |  8.9
+//     9,600 items, 3 disks                    22.8 | 14.1   16.9 | 11.6
 //
 // Edges:
 //  - FAR(t) after NEAR(t-1): the near items of t-1 are the only ones it may
