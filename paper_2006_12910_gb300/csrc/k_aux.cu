@@ -269,14 +269,13 @@ __global__ void __launch_bounds__(256) k_moments_f32(const __grid_constant__ Dom
             const W rs = vadd(r.h, r.l);
             W yr;
 #pragma unroll
-            for (int k = 0; k < N; ++k) {
-                rho[m * N + k] = K::get(rs, k);
-                plain[m * N + k] = K::get(rs, k) > 1e-30f && K::get(rs, k) < 1e30f;
-                K::set(yr, k, rcp_rho<float>(K::get(rs, k)));
-            }
+            for (int k = 0; k < N; ++k) K::set(yr, k, rcp_rho<float>(K::get(rs, k)));
             const W vx = velocity(sub(a, b), r, yr, P.gx2), vy = velocity(sub(c, d), r, yr, P.gy2);
+            const W big = vfma(vx, vx, vfma(vy, vy, rs));  // not below 1e30 when any of them leaves the range
 #pragma unroll
             for (int k = 0; k < N; ++k) {
+                rho[m * N + k] = K::get(rs, k);
+                plain[m * N + k] = K::get(rs, k) > 1e-30f && K::get(big, k) < 1e30f;
                 ux[m * N + k] = K::get(vx, k);
                 uy[m * N + k] = K::get(vy, k);
             }
@@ -435,7 +434,7 @@ static cudaError_t launch_moments_f32(const DomDev& D, const void* arena, const 
     auto pair = [](double v) { return FF{(float)v, (float)(v - (double)(float)v)}; };
     MomPrm P = {pair(D.rho0), pair(0.5 * D.gx), pair(0.5 * D.gy), 0, 1.0f};
     const int sh = 1086 - D.fix.e0;  // units of 2^-sh
-    if (D.fix.on && sh > 0 && sh < 120) {
+    if (D.fix.on && sh > 0 && sh < 120 && std::fabs(D.gx) < 1e30 && std::fabs(D.gy) < 1e30) {
         P.e0 = D.fix.e0;
         P.unit = std::ldexp(1.0f, -sh);
     }
