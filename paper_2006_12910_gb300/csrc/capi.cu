@@ -683,6 +683,16 @@ int ensure_stage(lbm_ctx* c, size_t bytes) {
     return LBM_OK;
 }
 
+// Marks, near-item counts and side-change tags of no step: before particles are
+// set up.  A tag of another run with the stamp of a step to come would send its
+// node's moments into a slot of lists it does not know.
+int clear_marks(lbm_ctx* c) {
+    CKC(c, cudaMemsetAsync(c->mark, 0xff, sizeof(int32_t) * 3 * std::max<int64_t>(1, c->total_items), c->stream));
+    CKC(c, cudaMemsetAsync(c->near_cnt, 0, sizeof(int32_t) * 3, c->stream));
+    CKC(c, cudaMemsetAsync(c->fliptag, 0xff, sizeof(int64_t) * 2 * std::max<size_t>(1, c->node_bytes), c->stream));
+    return LBM_OK;
+}
+
 // Solid bytes of one domain as the kernels read them, from its host mask.
 std::vector<uint8_t> pitched_solid(const lbm_ctx* c, int dom) {
     const DomDev& D = c->hd[dom];
@@ -1049,8 +1059,7 @@ int lbm_add_particles(lbm_ctx* c, int dom, int n, const lbm_particle* p) {
     // flips) and mark the work items near the particles for this step, then
     // what every step expects to find: the rasterisation of the next step
     // with its side changes and marks, and the Eq. MP2 sums of this step
-    CKC(c, cudaMemsetAsync(c->mark, 0xff, sizeof(int32_t) * 3 * std::max<int64_t>(1, c->total_items), c->stream));
-    CKC(c, cudaMemsetAsync(c->near_cnt, 0, sizeof(int32_t) * 3, c->stream));
+    if ((r = clear_marks(c))) return r;
     CKC(c, launch_particle_step(c->kind, part_args(c, c->cur), PL_RASTER | PL_MARK, c->stream));
     CKC(c, launch_particle_step(c->kind, part_args(c, c->cur), PL_SETUP_R, c->stream));
     CKC(c, launch_particle_step(c->kind, part_args(c, c->cur), PL_LJ, c->stream));
@@ -1434,8 +1443,7 @@ int lbm_load(lbm_ctx* c, const char* path) {
         c->np_active = np_total;
         c->steps = h.steps;  // the set-up launches take the step's parity from it
         CKC(c, cudaMemcpy(c->dd, c->hd.data(), sizeof(DomDev) * c->ndom, cudaMemcpyHostToDevice));
-        CKC(c, cudaMemset(c->mark, 0xff, sizeof(int32_t) * 3 * std::max<int64_t>(1, c->total_items)));
-        CKC(c, cudaMemset(c->near_cnt, 0, sizeof(int32_t) * 3));
+        if ((r = clear_marks(c))) return r;
         CKC(c, launch_particle_step(c->kind, part_args(c, c->cur), PL_MARK, c->stream));
         CKC(c, launch_particle_step(c->kind, part_args(c, c->cur), PL_SETUP_R, c->stream));
         CKC(c, launch_particle_step(c->kind, part_args(c, c->cur), PL_LJ, c->stream));
