@@ -112,6 +112,7 @@ struct lbm_ctx {
     int64_t* fliptag = nullptr;          // [2][nodes], copy by the parity of the tag's step
     double* ljf = nullptr;               // [2][np_slots][4]: Eq. MP2 force and torque, copy by step parity
     double* flipmom = nullptr;           // [2][flips_total][3]
+    uint32_t* fliplink = nullptr;        // [2][flips_total]
     int64_t near_grid = 1;
     bool any_lj = false;                 // some domain has an Eq. MP2 force
     LjEntry* lj_tab = nullptr;           // [ndom][LJ_TAB]
@@ -415,6 +416,7 @@ PartArgs part_args(lbm_ctx* c, int cur) {
     a.flipmom = c->flipmom;
     a.fliptag = c->fliptag;
     a.fliptag_stride = (int64_t)std::max<size_t>(1, c->node_bytes);
+    a.fliplink = c->fliplink;
     a.ljf = c->ljf;
     a.st = c->pst;
     a.np = c->np_slots;
@@ -465,6 +467,7 @@ cudaError_t enqueue_stream_collide(lbm_ctx* c, int cur, cudaStream_t s, int bloc
     a.near_cnt = c->near_cnt;
     a.fliptag = c->fliptag;
     a.fliptag_stride = (int64_t)std::max<size_t>(1, c->node_bytes);
+    a.fliplink = c->fliplink;
     a.flipmom = c->flipmom;
     a.dom0 = c->hd[0];
     return launch_stream_collide(c->kind, c->noise, c->pl, a, block, grid, c->grid_mode == 2 ? c->stages : 0, s, pdl);
@@ -728,10 +731,10 @@ int check_dom(lbm_ctx* c, int dom) {
 }
 
 void free_particles(lbm_ctx* c) {
-    cudaFree(c->pstate); cudaFree(c->pst); cudaFree(c->flipmom);
+    cudaFree(c->pstate); cudaFree(c->pst); cudaFree(c->flipmom); cudaFree(c->fliplink);
     cudaFree(c->links); cudaFree(c->nlinks); cudaFree(c->flips); cudaFree(c->nflips); cudaFree(c->diag);
     cudaFree(c->ljf);
-    c->pstate = nullptr; c->pst = nullptr; c->flipmom = nullptr;
+    c->pstate = nullptr; c->pst = nullptr; c->flipmom = nullptr; c->fliplink = nullptr;
     c->links = c->nlinks = c->flips = c->nflips = nullptr;
     c->diag = nullptr;
     c->ljf = nullptr;
@@ -1037,6 +1040,7 @@ int lbm_add_particles(lbm_ctx* c, int dom, int n, const lbm_particle* p) {
     const size_t ns = c->np_slots;
     CKC(c, dev_malloc(&c->pstate, sizeof(PartState) * 2 * ns));
     CKC(c, dev_malloc(&c->flipmom, sizeof(double) * 2 * 3 * std::max<int64_t>(fo, 1)));
+    CKC(c, dev_malloc(&c->fliplink, sizeof(int32_t) * 2 * std::max<int64_t>(fo, 1)));
     CKC(c, dev_malloc(&c->pst, sizeof(PartStatic) * ns));
     CKC(c, dev_malloc(&c->links, sizeof(int32_t) * 2 * std::max<int64_t>(lo, 1)));
     CKC(c, dev_malloc(&c->flips, sizeof(int32_t) * 2 * std::max<int64_t>(fo, 1)));
@@ -1418,6 +1422,7 @@ int lbm_load(lbm_ctx* c, const char* path) {
         c->hstate = s;
         CKC(c, dev_malloc(&c->pstate, sizeof(PartState) * 2 * ns));
         CKC(c, dev_malloc(&c->flipmom, 2 * 8 * fm.size()));
+        CKC(c, dev_malloc(&c->fliplink, 2 * 4 * F.size()));
         CKC(c, cudaMemset(c->flipmom, 0, 2 * 8 * fm.size()));
         CKC(c, dev_malloc(&c->pst, sizeof(PartStatic) * ns));
         CKC(c, dev_malloc(&c->links, 2 * 4 * L.size()));

@@ -1399,9 +1399,14 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(c
             if (fex < st.flip_cap) {
                 const int64_t idx = st.flip_off + fex;
                 flips[idx] = (node << 1) | (int)((r >> 10) & 1u);
-                // the stream-collide pass of this step leaves this node's moments in flipmom[slot]
+                // the stream-collide pass of this step leaves this node's moments in
+                // flipmom[slot], and in that of another disk that tagged it before
                 const int64_t slot = (int64_t)wpar * a.flips_total + idx;
-                a.fliptag[(int64_t)((t + 1) & 1) * a.fliptag_stride + D.node_off + node] = stamp | (uint32_t)slot;
+                const int64_t old = (int64_t)atomicExch(
+                    reinterpret_cast<unsigned long long*>(a.fliptag + (int64_t)((t + 1) & 1) * a.fliptag_stride +
+                                                          D.node_off + node),
+                    (unsigned long long)(stamp | (uint32_t)slot));
+                a.fliplink[slot] = (int32_t)(old >> 32) == (int32_t)(t + 1) ? (uint32_t)old : NO_SLOT;
             }
             ++fex;
         }

@@ -8,6 +8,7 @@
 
 namespace lbmk {
 
+constexpr uint32_t NO_SLOT = 0xffffffffu;
 struct StreamArgs {
     DomDev dom0;              // copy of doms[0] in the launch parameters (read when ndom == 1)
     const DomDev* doms;
@@ -32,9 +33,12 @@ struct StreamArgs {
     // Nodes that change side this step: a node whose tag carries step + 1
     // gets rho, sum f* e_x, sum f* e_y of its new populations written to
     // flipmom[3 * slot] (only work items near particles are looked at).  The
-    // tags of stamp s are in copy (s & 1), fliptag_stride nodes apart.
+    // tags of stamp s are in copy (s & 1), fliptag_stride nodes apart.  Where
+    // one disk uncovers the node and another covers it, fliplink[slot] is the
+    // other disk's slot (else NO_SLOT).
     const int64_t* fliptag;
     int64_t fliptag_stride;
+    const uint32_t* fliplink;
     double* flipmom;
     // Limit of the staged kernel's stage waits in global-timer nanoseconds
     // (1e9 by default; 0 makes every stage wait report expiry at once).
@@ -112,6 +116,7 @@ struct PartArgs {
     double* flipmom;           // [2][flips_total][3]: rho, sum f* e_x, sum f* e_y at the step of use
     int64_t* fliptag;          // [2][nodes]: (step << 32) | flip slot, copy (step & 1), for the stream-collide pass
     int64_t fliptag_stride;
+    uint32_t* fliplink;        // [2][flips_total]: see StreamArgs
     double* ljf;               // [2][np][4]: Eq. MP2 force x, y and torque on each particle at step s, copy (s & 1)
     double* diag;              // np * DIAG_N
     unsigned* err;

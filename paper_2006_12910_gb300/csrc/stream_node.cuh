@@ -139,7 +139,6 @@ __device__ __noinline__ void flip_moments(const StreamArgs& a, const DomDev& D, 
     const int64_t ni = (int64_t)y * D.pitch + x;
     const int64_t tag = a.fliptag[(int64_t)(stamp & 1) * a.fliptag_stride + D.node_off + ni];
     if ((int32_t)(tag >> 32) != stamp) return;
-    const uint32_t slot = (uint32_t)tag;
     double r = 0.0, jx = 0.0, jy = 0.0;
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
@@ -149,9 +148,12 @@ __device__ __noinline__ void flip_moments(const StreamArgs& a, const DomDev& D, 
         jx += v * cx(i);
         jy += v * cy(i);
     }
-    a.flipmom[3 * (int64_t)slot + 0] = r;
-    a.flipmom[3 * (int64_t)slot + 1] = jx;
-    a.flipmom[3 * (int64_t)slot + 2] = jy;
+#pragma unroll 1
+    for (uint32_t slot = (uint32_t)tag; slot != NO_SLOT; slot = a.fliplink[slot]) {
+        a.flipmom[3 * (int64_t)slot + 0] = r;
+        a.flipmom[3 * (int64_t)slot + 1] = jx;
+        a.flipmom[3 * (int64_t)slot + 2] = jy;
+    }
 }
 
 // Boundary nodes of a special chunk (fl: its flag words), before the collision:
