@@ -94,8 +94,9 @@ __device__ __forceinline__ bool collide_fix(const double (&f)[9], double (&out)[
     const uint32_t rhi = (uint32_t)((uint64_t)rho >> 32);
     ok = ok && rhi - 0x08800000u < 0x40000000u - 0x08800000u && (uint32_t)(mx >> 32) + 0x07FFFFF0u < 0x0FFFFFE0u &&
          (uint32_t)(my >> 32) + 0x07FFFFF0u < 0x0FFFFFE0u;
-    // y = 2^62 / rho in units of 2^-60: the FP32 reciprocal (error e below 2^-21)
-    // times 1 + e + e^2
+    // y = 2^62 / rho in units of 2^-60: y0, the hardware's FP32 reciprocal of the
+    // leading 32 bits, is off by e = 1 - rho y0 (below 2^-21); 1 / rho is y0 times
+    // the geometric series 1 / (1 - e), here 1 + e + e^2 (e^3 < 2^-63)
     const uint32_t y0 = __float2uint_rz(rcp_rho<float>((float)rhi) * 288230376151711744.0f);  // 2^58
     const int64_t e = (1ll << 60) - (int64_t)((((uint64_t)rhi * y0) << 2) + (((uint64_t)(uint32_t)rho * y0) >> 30));
     const int32_t eh = (int32_t)(e >> 16);

@@ -191,7 +191,8 @@ __device__ __forceinline__ FF pair_of(int64_t x) {
     return FF{s.h, __fadd_rn(s.l, c)};
 }
 // j / r - g2 (the velocity (j - r g / 2) / r) from the pairs, y about 1 / r:
-// the quotient's first digit and the remainder's, then the body-force term.
+// the quotient of two pairs (T. J. Dekker, Numer. Math. 18 (1971) 224) with y for
+// the divisions, a first digit and the remainder's, then the body-force term.
 template <class W>
 __device__ __forceinline__ W velocity(FFW<W> j, FFW<W> r, W y, FF g2) {
     typedef Vec<W> K;

@@ -159,12 +159,6 @@ __device__ __forceinline__ bool inside_f(const DomDev& D, const DiskF& k, int xu
     return inside_exact(D, k, xu, yu, wrapped);
 }
 
-template <class S>
-__device__ __forceinline__ double full_pop(const typename S::T* base, const DomDev& D, int i, int64_t ni) {
-    const double v = (double)to_a(base[(int64_t)i * D.plane + ni], (typename S::A)D.inv_scale);
-    return S::SHIFT ? v + wgt(i) * D.rho0 : v;
-}
-
 // Exclusive block scan of small non-negative counts; returns the block total.
 __device__ __noinline__ int block_scan(int c, int* sh_warp, int& excl) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;

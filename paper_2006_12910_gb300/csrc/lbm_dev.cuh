@@ -112,8 +112,7 @@ struct StF32S {
     static constexpr int MINB = 5, MINB_EXT = 4;
 };
 // Half-precision kinds take 8-byte vectors (4 nodes per lane): the register
-// footprint of an FP32 lane, so five CTAs fit per SM, and chunks near solids
-// store 4 rather than 8 nodes one by one.
+// footprint of an FP32 lane, so five CTAs fit per SM.
 struct StF16S {
     typedef __half T; typedef float A;
     static constexpr int V = 4; static constexpr bool SHIFT = true; static constexpr bool SCALED = true;
@@ -478,57 +477,50 @@ template <> __device__ __forceinline__ double rcp_rho<double>(double r) { return
 // c = 3 xi A^(n-1), is convex for n < 1 and concave for n > 1, so Newton from
 // the bracket end where g > 0 (n < 1) or g < 0 (n > 1) converges monotonically.
 // ---------------------------------------------------------------------------
-// FP32: the hardware base-2 logarithm (x > 0 here: a strain or a relaxation
-// time) and a division by the fast reciprocal inside the Newton steps, whose
-// fixed point (and so the converged tau*) does not depend on how a step is
-// rounded; FP64 keeps the exact operations.
-template <typename A> __device__ __forceinline__ A powa(A x, A e);
-template <> __device__ __forceinline__ float powa<float>(float x, float e) { return exp2f(e * __log2f(x)); }
-template <> __device__ __forceinline__ double powa<double>(double x, double e) { return exp2(e * log2(x)); }
-template <typename A> __device__ __forceinline__ A divn(A a, A b);
-template <> __device__ __forceinline__ float divn<float>(float a, float b) { return __fdividef(a, b); }
-template <> __device__ __forceinline__ double divn<double>(double a, double b) { return a / b; }
-
-template <typename A>
-__device__ __forceinline__ A solve_tau_pl(A Astr, const ExtPrm<A>& P) {
-    const A n = P.n, tmin = P.tmin, tmax = P.tmax;
+// FP64: one node, exact operations, converged to 10^-15.
+__device__ __forceinline__ double solve_tau_f64(double astr, const ExtPrm<double>& P) {
+    const double n = P.n, tmin = P.tmin, tmax = P.tmax;
     if (P.n_is_one) {
-        A t = (A)0.5 + (A)3.0 * P.xi;
+        const double t = 0.5 + 3.0 * P.xi;
         return t < tmin ? tmin : (t > tmax ? tmax : t);
     }
-    if (!(Astr > (A)0)) return n < (A)1 ? tmax : tmin;
-    const A om = (A)1 - n;
-    const A c = (A)3.0 * P.xi * powa<A>(Astr, n - (A)1);
-    if (tmin - (A)0.5 - c * P.tmin_pow >= (A)0) return tmin;
-    if (tmax - (A)0.5 - c * P.tmax_pow <= (A)0) return tmax;
-    A t = n < (A)1 ? tmax : tmin;
-    const A tol = sizeof(A) == 4 ? (A)2e-7 : (A)1e-15;
+    if (!(astr > 0.0)) return n < 1.0 ? tmax : tmin;
+    const double om = 1.0 - n;
+    const double c = 3.0 * P.xi * exp2((n - 1.0) * log2(astr));
+    if (tmin - 0.5 - c * P.tmin_pow >= 0.0) return tmin;
+    if (tmax - 0.5 - c * P.tmax_pow <= 0.0) return tmax;
+    double t = n < 1.0 ? tmax : tmin;
 #pragma unroll 1
     for (int it = 0; it < 60; ++it) {
-        const A p = powa<A>(t, om);
-        const A g = t - (A)0.5 - c * p;
-        const A dg = (A)1 - divn<A>(c * om * p, t);
-        A tn = t - divn<A>(g, dg);
+        const double p = exp2(om * log2(t));
+        const double g = t - 0.5 - c * p;
+        const double dg = 1.0 - c * om * p / t;
+        double tn = t - g / dg;
         tn = tn < tmin ? tmin : (tn > tmax ? tmax : tn);
-        const A dt = tn - t;
+        const double dt = tn - t;
         t = tn;
-        if (fabs(dt) <= tol * t) break;
+        if (fabs(dt) <= 1e-15 * t) break;
     }
     return t;
 }
-
-// tau* of NN nodes.  FP32: the iteration of solve_tau_pl on all of them in step,
-// so that their logarithms, exponentials and divisions overlap and a warp runs
-// as many iterations as its slowest node needs once, not node after node
-// (power law n = 0.75, 2048x1024 shifted FP32: 36.4 -> 30.8 us a step).  Every
-// node takes exactly the values solve_tau_pl gives it: where the strain is
-// small a last-place difference of tau* grows by 10^3 within 100 steps.  (Newton
-// from a near start, three evaluations a node, took 27.0 us and lost that.)
 template <int NN>
 __device__ __forceinline__ void solve_taus(const double (&astr)[NN], const ExtPrm<double>& P, double (&tau)[NN]) {
 #pragma unroll
-    for (int k = 0; k < NN; ++k) tau[k] = solve_tau_pl<double>(astr[k], P);
+    for (int k = 0; k < NN; ++k) tau[k] = solve_tau_f64(astr[k], P);
 }
+
+// FP32: the hardware base-2 logarithm (x > 0 here: a strain or a relaxation
+// time).
+__device__ __forceinline__ float pow_f32(float x, float e) { return exp2f(e * __log2f(x)); }
+
+// FP32: the same iteration on NN nodes in step, with the fast division and to
+// 2 10^-7, so that their logarithms, exponentials and divisions overlap and a
+// warp runs as many iterations as its slowest node needs once, not node after
+// node (power law n = 0.75, 2048x1024 shifted FP32: 36.4 -> 30.8 us a step).  A
+// node's values do not depend on the others in step with it; where the strain
+// is small a last-place difference of tau* grows by 10^3 within 100 steps, so
+// the order of its roundings is kept.  (Newton from a near start, three
+// evaluations a node, took 27.0 us and lost that.)
 template <int NN>
 __device__ __forceinline__ void solve_taus(const float (&astr)[NN], const ExtPrm<float>& P, float (&tau)[NN]) {
     const float n = P.n, tmin = P.tmin, tmax = P.tmax, om = 1.0f - n;
@@ -536,7 +528,7 @@ __device__ __forceinline__ void solve_taus(const float (&astr)[NN], const ExtPrm
     bool open[NN], any = false;
 #pragma unroll
     for (int k = 0; k < NN; ++k) {
-        c[k] = __fmul_rn(3.0f * P.xi, powa<float>(astr[k], n - 1.0f));
+        c[k] = __fmul_rn(3.0f * P.xi, pow_f32(astr[k], n - 1.0f));
         const bool low = astr[k] > 0.0f ? tmin - 0.5f - c[k] * P.tmin_pow >= 0.0f : n >= 1.0f;
         const bool high = astr[k] > 0.0f ? tmax - 0.5f - c[k] * P.tmax_pow <= 0.0f : n < 1.0f;
         if (P.n_is_one) tau[k] = fminf(fmaxf(0.5f + 3.0f * P.xi, tmin), tmax);
@@ -549,7 +541,7 @@ __device__ __forceinline__ void solve_taus(const float (&astr)[NN], const ExtPrm
         any = false;
         float p[NN];
 #pragma unroll
-        for (int k = 0; k < NN; ++k) p[k] = powa<float>(tau[k], om);
+        for (int k = 0; k < NN; ++k) p[k] = pow_f32(tau[k], om);
 #pragma unroll
         for (int k = 0; k < NN; ++k) {
             const float t = tau[k];
