@@ -175,12 +175,20 @@ __device__ __forceinline__ void load_pop(__nv_bfloat16& v, const void* p) {
     asm volatile("ld.global.u16 %0, [%1];" : "=h"(u) : "l"(p));
     v = __ushort_as_bfloat16(u);
 }
+// The same past the L1, for data read once (the moments of 2048x1024 nodes in FP32,
+// launches back to back: 17.6 us, 19.3 through the L1, 17.6 with __ldg).
+__device__ __forceinline__ void load_once(uint4& v, const void* p) {
+    asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+}
+__device__ __forceinline__ void load_once(uint2& v, const void* p) {
+    asm volatile("ld.global.cg.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+}
 // Vector load of NV consecutive elements: one 8- or 16-byte access.
 template <class S, int NV>
 __device__ __forceinline__ void load_vec(const typename S::T* p, typename S::A (&out)[NV], typename S::A inv) {
     typedef typename VecOf<NV * sizeof(typename S::T)>::type VT;
     union { VT u; typename S::T t[NV]; } r;
-    load_pop(r.u, p);
+    load_once(r.u, p);
 #pragma unroll
     for (int k = 0; k < NV; ++k) out[k] = to_a(r.t[k], inv);
 }
