@@ -9,10 +9,10 @@
 // rho0 2^s in [2^60, 2^61) hold them with more digits than FP64 does: an addition
 // is exact, a product of two such numbers is good to 1.3 units (three 32 x 32 ->
 // 64-bit multiplies), where FP64 rounds the density to 2^8 units and the
-// populations to 2^2 .. 2^6.  About 700 integer instructions a node: 281 -> 73 us
+// populations to 2^2 .. 2^6.  About 700 integer instructions a node: 281 -> 70 us
 // a step at 2048x1024 (64 % issue, ALU pipe 63 %; 32 warps of 64 registers per
 // SM, one node a lane; two nodes a lane held 12 warps and took 92 us), 256x64
-// 7.75 -> 3.2 us.  One collision is off by 1.16e-17 rho0 rms a population, FP64
+// 7.75 -> 3.0 us.  One collision is off by 1.16e-17 rho0 rms a population, FP64
 // arithmetic by 2.1e-17 (exact rational arithmetic as the measure).
 //
 // A node outside the range of the format is left to the FP64 collision: a

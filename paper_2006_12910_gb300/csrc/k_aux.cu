@@ -209,9 +209,9 @@ __device__ __forceinline__ W velocity(FFW<W> j, FFW<W> r, W y, FF g2) {
 // another without the launch gap; each still waits for the one before it.
 // Bound by HBM (FP32 stores: 70 % of the copy rate) and, for the half-precision
 // stores, by arithmetic.  Measured, launches back to back, against FP64
-// sums and divisions a node at a time: 2048x1024 shifted FP32 260 -> 18.2 us,
-// FP16 265 -> 13.5, FP64 191 -> 33 (exact sums in the fixed-point
-// format of the collision); 96 ensemble domains (96 launches) 1812 -> 344 or
+// sums and divisions a node at a time: 2048x1024 shifted FP32 260 -> 17.4 us,
+// FP16 265 -> 12.7, FP64 191 -> 29.7 (exact sums in the fixed-point
+// format of the collision); 96 ensemble domains (96 launches) 1812 -> 410 or
 // less; 4096x2048 1023 -> 72.
 template <class S>
 __host__ __device__ constexpr int moment_chunk() { return sizeof(typename S::T) == 8 ? 2 : 4; }

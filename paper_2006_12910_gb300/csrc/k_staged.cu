@@ -19,7 +19,7 @@
 // on as the register kernel does (form_chunk, patch_chunk, finish_chunk; equal
 // results).  The register kernel is the default: a bulk copy costs its SM about
 // 40 cycles here, and nine small ones an item (1 KB a row at most) made this
-// kernel 30 us against 26.5 (FP32, 2048x1024) and 20.6 against 14.4 (FP16).
+// kernel 30 us against 26.4 (FP32, 2048x1024) and 20.6 against 14.7 (FP16).
 // Open ends and corners read their sources from global memory.  Every mbarrier
 // wait is bounded (about one second by the global timer); a wait that runs
 // out sets ERR_TIMEOUT, waits (bounded again, always by the full second) for

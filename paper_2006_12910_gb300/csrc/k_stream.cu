@@ -22,8 +22,8 @@
 // ragged last chunk treats the padding beyond the row as solid nodes.
 //
 // Bounds: FP32 stores by HBM and L2 (2048x1024 porous geometry, one graph:
-// 27.5 -> 26.5 us a step; 4096x2048 103.6 -> 103.2, 5.9 TB/s); half-precision
-// stores by latency and issue (18.7 -> 14.4 us); noise and tau* by arithmetic.
+// 27.5 -> 26.4 us a step; 4096x2048 103.6 -> 101.9, 5.9 TB/s); half-precision
+// stores by latency and issue (18.7 -> 14.7 us); noise and tau* by arithmetic.
 #include "stream_node.cuh"
 
 namespace lbmk {

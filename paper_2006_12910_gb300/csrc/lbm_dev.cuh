@@ -288,7 +288,7 @@ __device__ __forceinline__ W neg_sqrt(W nx, W y) {
 // relative error of ln u at most 1.37 x 2^-24.  The noise variant is bound by
 // arithmetic: in packed pairs this and the square root below take half the
 // instructions of logf and sqrtf (2048x1024 shifted FP32 with noise: 37.5 ->
-// 29.5 us a step, 1,803 -> 1,230 instructions an item with the packed
+// 28.7 us a step, 1,803 -> 1,230 instructions an item with the packed
 // collision).  Against 64 bits the noise of one node is off by 1.620e-7 of its
 // rms (1.625e-7 with logf and sqrtf), set by the hardware sine and cosine.
 template <class W>

@@ -26,6 +26,7 @@ def test_velocities_beyond_fp32(store):
     f[[0, 1, 3], 2, 8] = 1.0, 2e38, -2e38
     ctx.set_populations(f)
     out = [torch.full((ny, nx), float("nan"), device="cuda") for _ in range(3)]
+    torch.cuda.synchronize()
     ctx.moments_device(*out)
     ctx.sync()
     with np.errstate(over="ignore"):
