@@ -120,7 +120,9 @@ int lbm_set_geometry(lbm_ctx* ctx, int dom, const uint8_t* solid);
 
 /* Add n particles to domain dom (copied) and rasterise them (Sec. 3, Fig. 1:
  * a node belongs to a particle when strictly inside its disk).  Particles
- * must not overlap each other.  Total per domain <= max_particles. */
+ * must not overlap each other.  Total per domain <= max_particles.  When the
+ * device memory for them cannot be had (LBM_E_NOMEM) the context goes on
+ * without any particles. */
 int lbm_add_particles(lbm_ctx* ctx, int dom, int n, const lbm_particle* p);
 
 /* Replace the populations f*(t) of domain dom with host FP64 values

@@ -740,6 +740,14 @@ void free_particles(lbm_ctx* c) {
     c->ljf = nullptr;
 }
 
+// No particles in any domain (the device descriptors are uploaded with the next ones).
+void drop_particles(lbm_ctx* c) {
+    free_particles(c);
+    for (auto& D : c->hd) D.np = 0;
+    for (auto& st : c->hst) st.dom = -1;
+    c->np_active = 0;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1036,27 +1044,39 @@ int lbm_add_particles(lbm_ctx* c, int dom, int n, const lbm_particle* p) {
         lo += st.link_cap;
         fo += st.flip_cap;
     }
+    // Without its arrays the context can hold no particles: they go, on failure.
+#define CKP(call)                                                                                  \
+    do {                                                                                           \
+        cudaError_t e_ = (call);                                                                   \
+        if (e_ != cudaSuccess) {                                                                   \
+            drop_particles(c);                                                                     \
+            return fail(c, e_ == cudaErrorMemoryAllocation ? LBM_E_NOMEM : LBM_E_CUDA,             \
+                        std::string(#call) + ": " + cudaGetErrorString(e_) + " (particles removed)"); \
+        }                                                                                          \
+    } while (0)
     free_particles(c);
+    c->graph_dirty = true;  // the step graphs hold the old arrays
     const size_t ns = c->np_slots;
-    CKC(c, dev_malloc(&c->pstate, sizeof(PartState) * 2 * ns));
-    CKC(c, dev_malloc(&c->flipmom, sizeof(double) * 2 * 3 * std::max<int64_t>(fo, 1)));
-    CKC(c, dev_malloc(&c->fliplink, sizeof(int32_t) * 2 * std::max<int64_t>(fo, 1)));
-    CKC(c, dev_malloc(&c->pst, sizeof(PartStatic) * ns));
-    CKC(c, dev_malloc(&c->links, sizeof(int32_t) * 2 * std::max<int64_t>(lo, 1)));
-    CKC(c, dev_malloc(&c->flips, sizeof(int32_t) * 2 * std::max<int64_t>(fo, 1)));
-    CKC(c, dev_malloc(&c->nlinks, sizeof(int32_t) * 2 * ns));
-    CKC(c, dev_malloc(&c->nflips, sizeof(int32_t) * 2 * ns));
-    CKC(c, dev_malloc(&c->diag, sizeof(double) * DIAG_N * ns));
-    CKC(c, dev_malloc(&c->ljf, sizeof(double) * 2 * 4 * ns));
-    CKC(c, cudaMemset(c->ljf, 0, sizeof(double) * 2 * 4 * ns));
-    CKC(c, cudaMemset(c->flipmom, 0, sizeof(double) * 2 * 3 * std::max<int64_t>(fo, 1)));
-    CKC(c, cudaMemset(c->nlinks, 0, sizeof(int32_t) * 2 * ns));
-    CKC(c, cudaMemset(c->nflips, 0, sizeof(int32_t) * 2 * ns));
-    CKC(c, cudaMemset(c->diag, 0, sizeof(double) * DIAG_N * ns));
-    CKC(c, cudaMemcpy(c->pstate, c->hstate.data(), sizeof(PartState) * ns, cudaMemcpyHostToDevice));
-    CKC(c, cudaMemcpy(c->pstate + ns, c->hstate.data(), sizeof(PartState) * ns, cudaMemcpyHostToDevice));
-    CKC(c, cudaMemcpy(c->pst, c->hst.data(), sizeof(PartStatic) * ns, cudaMemcpyHostToDevice));
-    CKC(c, cudaMemcpy(c->dd + dom, &D, sizeof(DomDev), cudaMemcpyHostToDevice));
+    CKP(dev_malloc(&c->pstate, sizeof(PartState) * 2 * ns));
+    CKP(dev_malloc(&c->flipmom, sizeof(double) * 2 * 3 * std::max<int64_t>(fo, 1)));
+    CKP(dev_malloc(&c->fliplink, sizeof(int32_t) * 2 * std::max<int64_t>(fo, 1)));
+    CKP(dev_malloc(&c->pst, sizeof(PartStatic) * ns));
+    CKP(dev_malloc(&c->links, sizeof(int32_t) * 2 * std::max<int64_t>(lo, 1)));
+    CKP(dev_malloc(&c->flips, sizeof(int32_t) * 2 * std::max<int64_t>(fo, 1)));
+    CKP(dev_malloc(&c->nlinks, sizeof(int32_t) * 2 * ns));
+    CKP(dev_malloc(&c->nflips, sizeof(int32_t) * 2 * ns));
+    CKP(dev_malloc(&c->diag, sizeof(double) * DIAG_N * ns));
+    CKP(dev_malloc(&c->ljf, sizeof(double) * 2 * 4 * ns));
+    CKP(cudaMemset(c->ljf, 0, sizeof(double) * 2 * 4 * ns));
+    CKP(cudaMemset(c->flipmom, 0, sizeof(double) * 2 * 3 * std::max<int64_t>(fo, 1)));
+    CKP(cudaMemset(c->nlinks, 0, sizeof(int32_t) * 2 * ns));
+    CKP(cudaMemset(c->nflips, 0, sizeof(int32_t) * 2 * ns));
+    CKP(cudaMemset(c->diag, 0, sizeof(double) * DIAG_N * ns));
+    CKP(cudaMemcpy(c->pstate, c->hstate.data(), sizeof(PartState) * ns, cudaMemcpyHostToDevice));
+    CKP(cudaMemcpy(c->pstate + ns, c->hstate.data(), sizeof(PartState) * ns, cudaMemcpyHostToDevice));
+    CKP(cudaMemcpy(c->pst, c->hst.data(), sizeof(PartStatic) * ns, cudaMemcpyHostToDevice));
+    CKP(cudaMemcpy(c->dd, c->hd.data(), sizeof(DomDev) * c->ndom, cudaMemcpyHostToDevice));
+#undef CKP
     c->links_total = lo;
     c->flips_total = fo;
     // rasterise every particle at its current position (no link exchange, no
@@ -1068,7 +1088,6 @@ int lbm_add_particles(lbm_ctx* c, int dom, int n, const lbm_particle* p) {
     CKC(c, launch_particle_step(c->kind, part_args(c, c->cur), PL_SETUP_R, c->stream));
     CKC(c, launch_particle_step(c->kind, part_args(c, c->cur), PL_LJ, c->stream));
     CKC(c, launch_particle_step(c->kind, part_args(c, c->cur), PL_LJ | PL_ADVANCE, c->stream));
-    c->graph_dirty = true;
     return sync_and_check(c);
 }
 
@@ -1406,6 +1425,7 @@ int lbm_load(lbm_ctx* c, const char* path) {
         if (!ok) return bail("truncated checkpoint");
     }
     fclose(fp);
+    c->graph_dirty = true;  // also when a later call fails: the step graphs hold the old arrays
     // geometry first (it rewrites solid nodes of the current arena), then the state
     for (int d = 0; d < c->ndom; ++d) {
         c->hd[d].np = 0;
