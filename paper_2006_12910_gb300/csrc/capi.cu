@@ -1009,10 +1009,30 @@ int lbm_add_particles(lbm_ctx* c, int dom, int n, const lbm_particle* p) {
         if ((D.flags & FLAG_PY) && 2 * q.R + 8 >= D.ny) return fail(c, LBM_E_INVAL, "particle too large for the periodic y extent");
     }
     CKC(c, cudaStreamSynchronize(c->stream));
-    // refresh the host shadow of the existing particle states
-    if (c->np_active > 0)
-        CKC(c, cudaMemcpy(c->hstate.data(), c->pstate + (c->steps & 1) * c->np_slots, sizeof(PartState) * c->np_slots,
+    // refresh the host shadow of the existing particle states, and keep the side
+    // changes of this step with their moments: the rasterisation below finds
+    // none, and the forces of this step need them
+    const int64_t par = c->steps & 1;
+    struct Changes {
+        int slot;
+        std::vector<int32_t> nodes;
+        std::vector<double> mom;
+    };
+    std::vector<Changes> kept;
+    if (c->np_active > 0) {
+        CKC(c, cudaMemcpy(c->hstate.data(), c->pstate + par * c->np_slots, sizeof(PartState) * c->np_slots,
                           cudaMemcpyDeviceToHost));
+        std::vector<int32_t> nf(c->np_slots);
+        CKC(c, cudaMemcpy(nf.data(), c->nflips + par * c->np_slots, sizeof(int32_t) * c->np_slots, cudaMemcpyDeviceToHost));
+        for (int s = 0; s < c->np_slots; ++s) {
+            if (c->hst[s].dom < 0 || nf[s] <= 0) continue;
+            const int64_t at = par * c->flips_total + c->hst[s].flip_off;
+            Changes k{s, std::vector<int32_t>(nf[s]), std::vector<double>(3 * (size_t)nf[s])};
+            CKC(c, cudaMemcpy(k.nodes.data(), c->flips + at, sizeof(int32_t) * k.nodes.size(), cudaMemcpyDeviceToHost));
+            CKC(c, cudaMemcpy(k.mom.data(), c->flipmom + 3 * at, sizeof(double) * k.mom.size(), cudaMemcpyDeviceToHost));
+            kept.push_back(std::move(k));
+        }
+    }
     const double pi = 3.14159265358979323846264338327950288;
     for (int i = 0; i < n; ++i) {
         const lbm_particle& q = p[i];
@@ -1088,7 +1108,15 @@ int lbm_add_particles(lbm_ctx* c, int dom, int n, const lbm_particle* p) {
     CKC(c, launch_particle_step(c->kind, part_args(c, c->cur), PL_SETUP_R, c->stream));
     CKC(c, launch_particle_step(c->kind, part_args(c, c->cur), PL_LJ, c->stream));
     CKC(c, launch_particle_step(c->kind, part_args(c, c->cur), PL_LJ | PL_ADVANCE, c->stream));
-    return sync_and_check(c);
+    r = sync_and_check(c);
+    for (const Changes& k : kept) {
+        const int64_t at = par * c->flips_total + c->hst[k.slot].flip_off;
+        const int32_t n_k = (int32_t)k.nodes.size();
+        CKC(c, cudaMemcpy(c->flips + at, k.nodes.data(), sizeof(int32_t) * k.nodes.size(), cudaMemcpyHostToDevice));
+        CKC(c, cudaMemcpy(c->flipmom + 3 * at, k.mom.data(), sizeof(double) * k.mom.size(), cudaMemcpyHostToDevice));
+        CKC(c, cudaMemcpy(c->nflips + par * c->np_slots + k.slot, &n_k, sizeof n_k, cudaMemcpyHostToDevice));
+    }
+    return r;
 }
 
 // Wait for the work queued so far and clear the sticky device error word:
