@@ -1139,6 +1139,8 @@ int lbm_set_populations(lbm_ctx* c, int dom, const double* f) {
     if (r) return r;
     CKC(c, cudaMemcpyAsync(c->d_stage, f, bytes, cudaMemcpyHostToDevice, c->stream));
     CKC(c, launch_import(c->kind, D, c->d_stage, c->f[c->cur], c->solid, c->stream));
+    // the covered / uncovered force of this step is that of the new populations
+    if (D.np > 0) CKC(c, launch_flip_moments(c->kind, part_args(c, c->cur), D.p0, D.np, c->stream));
     return sync_and_check(c);
 }
 

@@ -1412,6 +1412,31 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(c
     }
 }
 
+template <class S>
+__global__ void k_flip_moments(const __grid_constant__ PartArgs a, int p0) {
+    const int p = p0 + (int)blockIdx.x;
+    const PartStatic st = a.st[p];
+    const DomDev& D = a.doms[st.dom];
+    const typename S::T* base = static_cast<const typename S::T*>(a.arena) + D.off;
+    const int64_t at = (int64_t)a.par * a.flips_total + st.flip_off;
+    const int nf = a.nflips[(int64_t)a.par * a.np + p];
+    for (int l = threadIdx.x; l < nf; l += blockDim.x) {
+        const int64_t node = a.flips[at + l] >> 1;
+        double r = 0.0, jx = 0.0, jy = 0.0;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            double v = (double)to_a(base[(int64_t)i * D.plane + node], (typename S::A)D.inv_scale);
+            if (S::SHIFT) v += wgt(i) * D.rho0;
+            r += v;
+            jx += v * cx(i);
+            jy += v * cy(i);
+        }
+        a.flipmom[3 * (at + l) + 0] = r;
+        a.flipmom[3 * (at + l) + 1] = jx;
+        a.flipmom[3 * (at + l) + 2] = jy;
+    }
+}
+
 #define LBM_PDISPATCH(kind, CALL)                     \
     switch (kind) {                                   \
         case 0: { typedef StF64 S; CALL; } break;     \
@@ -1439,6 +1464,11 @@ static cudaError_t launch_part(const PartArgs& a, int modes, int role0, int grid
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k_particle_step<S, LO, HI>, a, modes, role0);
+}
+
+cudaError_t launch_flip_moments(int kind, const PartArgs& a, int p0, int np, cudaStream_t s) {
+    LBM_PDISPATCH(kind, (k_flip_moments<S><<<(unsigned)np, 128, 0, s>>>(a, p0)))
+    return cudaGetLastError();
 }
 
 cudaError_t launch_particle_step(int kind, const PartArgs& a, int modes, cudaStream_t s, bool pdl) {

@@ -161,6 +161,10 @@ constexpr int PL_SETUP_R = PL_RASTER | PL_MARK | PL_ADVANCE;
 // stream-collide pass after it is placed while the exchange completes.
 cudaError_t launch_particle_step(int kind, const PartArgs& a, int modes, cudaStream_t s, bool pdl = false);
 
+// Moments of the nodes that changed side for the current step, from the populations in a.arena,
+// of the np particles of one domain from slot p0 on (when the populations are replaced).
+cudaError_t launch_flip_moments(int kind, const PartArgs& a, int p0, int np, cudaStream_t s);
+
 // The thread's message for lbm_last_error(NULL) (capi.cu).
 void set_global_error(const char* msg);
 
