@@ -482,7 +482,7 @@ __global__ void __launch_bounds__(LO >= 2 ? BC_BLOCK : PBLOCK) k_particle_step(c
         //     c_k = 2 rho0 omega_k / c_s^2, a_k = (e_kx, e_ky, (r_b - r_c) x e_k);
         //     warp 4: covered / uncovered nodes.  The Eq. MP2 force at t was
         //     summed by role D two steps earlier (or at set-up).
-        //  2. thread 0: Eqs. MP5-MP6 with the force -Z X_mid of the moving
+        //  2. lanes of warp 0: Eqs. MP5-MP6 with the force -Z X_mid of the moving
         //     boundary, X_mid = (X(t) + X(t+1)) / 2: the SPD system
         //     (M + Z/2) X_mid = M X(t) + G/2 by its adjugate, X(t+1) = 2 X_mid - X(t).
         //  3. warps 0-3: the exchange of Eqs. MP7-MP8 with u_b(X_mid) on each
